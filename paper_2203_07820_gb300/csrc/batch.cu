@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <array>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <string>
 #include <vector>
@@ -31,7 +32,8 @@ struct SysStep {
   const double* Xp;
   double* Z;
   int64_t ldx, ldp, ldz, M;
-  int nc, ncol, active;
+  int nc, ncol;
+  int active;              // 1: dense cell products, 2: tensor-product form (its own launches)
   int cplx;                // real view of a complex block: the init is the k-point kernel's
   double alpha, s1, s2;
 };
@@ -52,6 +54,9 @@ struct dftfe_batch_s {
   std::vector<dftfe::bt::SysStep> host_steps;   // their host copy (kept until the next pass)
   // descriptors of the batched split-precision filter (device buffer and its host staging)
   dftfe::DevBuf mixed_desc;
+  // items and work lists of the FP64 tensor-product launches
+  dftfe::DevBuf sf_desc;
+  std::vector<uint8_t> sf_host;
   std::vector<uint8_t> mixed_host;
   // autotuner of the split-precision cell-product launches (dftfe_batch_autotune)
   bool autotune = false;
@@ -72,7 +77,7 @@ namespace dftfe {
 // same order as the single-system k_axpby_init
 __global__ void k_batch_axpby(const bt::SysStep* __restrict__ st) {
   const bt::SysStep& d = st[blockIdx.y];
-  if (!d.active || d.cplx) return;
+  if (d.active != 1 || d.cplx) return;
   const int64_t n = d.M * d.ncol;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = t / d.ncol;
@@ -91,7 +96,7 @@ __global__ void __launch_bounds__(256, 2) k_batch_cell(const bt::SysStep* __rest
   extern __shared__ double smem[];
   const bt::SysStep& d = st[wsys[blockIdx.x]];
   const int rbeg = (int)blockIdx.z * rows_per_split;
-  if (!d.active || (int)blockIdx.y * 32 >= d.ncol || rbeg >= d.nc) return;
+  if (d.active != 1 || (int)blockIdx.y * 32 >= d.ncol || rbeg >= d.nc) return;
   cell_fp64_wide_body(d.Hc, d.map, wcell[blockIdx.x], d.nc, d.X, d.ldx, d.Z, d.ldz, d.ncol, d.alpha,
                       (int)blockIdx.y, rbeg, min(d.nc, rbeg + rows_per_split), smem);
 }
@@ -123,9 +128,18 @@ static void cheb_coef(const dftfe_bounds& b, int k, double& sigma, double& alpha
 // One round = block j of every system.  The descriptors of every round and step are formed
 // on the host and uploaded before any launch, so the launches of the whole filter phase need
 // no host work in between and can be captured as one CUDA graph.
+// A launch of the tensor-product kernels over the systems of one FE degree and quadrature rule:
+// offsets into the uploaded items and work lists.
+struct SfLaunch {
+  const dftfe_mesh_s* mesh;
+  size_t item_off, cell_off, face_off;
+  int64_t ncell, nface;
+};
+
 struct RoundPlan {
   std::vector<int> nb;                       // real columns of block j (0: none / alone)
-  std::vector<int> alone;                    // blocks of at most 4 real columns: single filter
+  std::vector<int> alone;                    // dense blocks of at most 4 real columns: single filter
+  std::vector<std::vector<SfLaunch>> sf;     // per step
   std::vector<int> cur;                      // buffer holding the result after the last step
   std::vector<std::array<double*, 3>> buf;
   std::vector<std::array<int64_t, 3>> lds;
@@ -153,12 +167,17 @@ static void batch_filter(dftfe_batch bt, dftfe_batch_item* items) {
   DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_batch_cell, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh));
   // the two recurrence workspaces of each system, at the size of its widest block (all
   // rounds' descriptors point into them, so they must not be reallocated between rounds)
-  std::vector<double*> w1(ns, nullptr), w2(ns, nullptr);
+  std::vector<double*> w1(ns, nullptr), w2(ns, nullptr), face(ns, nullptr);
+  std::vector<sf::Item<double>> sf_items;
+  std::vector<int2> sf_work;
+  std::map<std::vector<int>, SfLaunch> sf_lists;      // work lists by the (system, columns) they cover
   for (int s = 0; s < ns; ++s) {
     const int cw = items[s].kpoint ? 2 : 1;
     const int widest = cw * std::min(items[s].block, items[s].ncol);
-    if (widest <= 4 || items[s].degree <= 0) continue;
     dftfe_ham h = bt->hams[s];
+    const bool sf = sf_applicable(h->mesh);
+    if ((widest <= 4 && !sf) || items[s].degree <= 0) continue;
+    if (sf) face[s] = (double*)ws_get(h, "sf_face", sizeof(double) * sf_face_elems(h->mesh, widest));
     w1[s] = (double*)ws_get(h, "cheb_w1", sizeof(double) * h->mesh->M * (size_t)widest);
     w2[s] = (double*)ws_get(h, "cheb_w2", sizeof(double) * h->mesh->M * (size_t)widest);
   }
@@ -176,13 +195,14 @@ static void batch_filter(dftfe_batch bt, dftfe_batch_item* items) {
       const int cw = items[s].kpoint ? 2 : 1;
       int nb = cw * std::min(items[s].block, items[s].ncol - j * items[s].block);
       if (nb <= 0 || items[s].degree <= 0) continue;
-      if (nb <= 4) {
+      if (nb <= 4 && !face[s]) {
         r.alone.push_back(s);
         continue;
       }
       r.nb[s] = nb;
       r.buf[s] = {items[s].X + (int64_t)cw * j * items[s].block, w1[s], w2[s]};
       r.lds[s] = {cw * items[s].ld, nb, nb};
+      if (face[s]) continue;
       r.maxtiles = std::max(r.maxtiles, (nb + 31) / 32);
       r.maxwork = std::max<int64_t>(r.maxwork, bt->hams[s]->mesh->M * nb);
     }
@@ -207,7 +227,7 @@ static void batch_filter(dftfe_batch bt, dftfe_batch_item* items) {
         d.M = h->mesh->M;
         d.nc = h->mesh->nc;
         d.ncol = r.nb[s];
-        d.active = 1;
+        d.active = face[s] ? 2 : 1;
         d.cplx = items[s].kpoint ? 1 : 0;
         d.alpha = alpha;
         d.s1 = s1;
@@ -215,7 +235,62 @@ static void batch_filter(dftfe_batch bt, dftfe_batch_item* items) {
         prev[s] = r.cur[s];
         r.cur[s] = out;
       }
+    // tensor-product launches: the systems still filtering, one launch per degree and rule
+    r.sf.resize(maxdeg);
+    for (int k = 1; k <= maxdeg; ++k) {
+      const bt::SysStep* dk = &bt->host_steps[(size_t)j * per_round + (size_t)(k - 1) * ns];
+      std::map<std::pair<int, int>, std::vector<int>> groups;
+      for (int s = 0; s < ns; ++s)
+        if (dk[s].active == 2) {
+          const auto* m = bt->hams[s]->mesh;
+          groups[{m->n1, m->vquad}].push_back(s);
+        }
+      for (auto& g : groups) {
+        std::vector<int> key;
+        for (int s : g.second) {
+          key.push_back(s);
+          key.push_back(dk[s].ncol);
+        }
+        auto it = sf_lists.find(key);
+        if (it == sf_lists.end()) {
+          SfLaunch L{bt->hams[g.second[0]]->mesh, 0, sf_work.size(), 0, 0, 0};
+          for (size_t q = 0; q < g.second.size(); ++q) {
+            const int64_t n = sf_cell_work64(bt->hams[g.second[q]]->mesh, dk[g.second[q]].ncol);
+            for (int64_t t = 0; t < n; ++t) sf_work.push_back(make_int2((int)q, (int)t));
+          }
+          L.ncell = (int64_t)(sf_work.size() - L.cell_off);
+          L.face_off = sf_work.size();
+          for (size_t q = 0; q < g.second.size(); ++q)
+            for (int64_t t = 0; t < bt->hams[g.second[q]]->mesh->Nc; ++t)
+              sf_work.push_back(make_int2((int)q, (int)t));
+          L.nface = (int64_t)(sf_work.size() - L.face_off);
+          it = sf_lists.emplace(key, L).first;
+        }
+        SfLaunch L = it->second;
+        L.item_off = sf_items.size();
+        for (int s : g.second) {
+          const bt::SysStep& d = dk[s];
+          // a complex block already holds its recurrence and k terms in Z
+          sf_items.push_back(sf_item64(bt->hams[s], face[s], d.X, d.ldx, d.cplx ? d.Z : d.Xp, d.cplx ? d.ldz : d.ldp,
+                                       d.Z, d.ldz, d.ncol, d.alpha, d.cplx ? 0.0 : d.s1, d.cplx ? 1.0 : d.s2));
+        }
+        r.sf[k - 1].push_back(L);
+      }
+    }
   }
+  const size_t sf_ib = (sf_items.size() * sizeof(sf::Item<double>) + 255) / 256 * 256;
+  bt->sf_host.resize(sf_ib + sf_work.size() * sizeof(int2));
+  if (!sf_items.empty()) {
+    std::memcpy(bt->sf_host.data(), sf_items.data(), sf_items.size() * sizeof(sf::Item<double>));
+    std::memcpy(bt->sf_host.data() + sf_ib, sf_work.data(), sf_work.size() * sizeof(int2));
+  }
+  if (bt->sf_host.size() > bt->sf_desc.bytes) DFTFE_CHECK_CUDA(cudaStreamSynchronize(bt->stream));
+  uint8_t* sf_dev = (uint8_t*)bt->sf_desc.get(bt->sf_host.size());
+  if (!bt->sf_host.empty())
+    DFTFE_CHECK_CUDA(cudaMemcpyAsync(sf_dev, bt->sf_host.data(), bt->sf_host.size(), cudaMemcpyHostToDevice,
+                                     bt->stream));
+  const auto* sf_ditems = reinterpret_cast<const sf::Item<double>*>(sf_dev);
+  const auto* sf_dwork = reinterpret_cast<const int2*>(sf_dev + sf_ib);
   // from pageable memory: the call returns once the data is staged, so the host descriptors
   // may be rewritten by the next pass
   DFTFE_CHECK_CUDA(cudaMemcpyAsync(dsteps, bt->host_steps.data(), sizeof(bt::SysStep) * bt->host_steps.size(),
@@ -237,7 +312,17 @@ static void batch_filter(dftfe_batch bt, dftfe_batch_item* items) {
           if (d.cplx)      // the recurrence terms, 1/2|k|^2, -i k.grad and the phased projectors
             kpoint_init_terms(bt->hams[s], d.X, d.ldx / 2, d.Xp, d.ldp / 2, d.Z, d.ldz / 2, d.ncol / 2, d.alpha,
                               d.s1, d.s2);
-          else
+          else if (d.active == 1)
+            nonlocal_add_fp64(bt->hams[s], d.X, d.ldx, d.Z, d.ldz, d.ncol, d.alpha);
+        }
+        for (const SfLaunch& L : r.sf[k - 1]) {
+          ProfScope ps(bt->hams[0], "batch_cell");
+          sf_launch64(bt->stream, bt->hams[0]->sm_count, L.mesh, sf::Item<double>{}, sf_ditems + L.item_off, sf_dwork + L.cell_off, L.ncell,
+                      sf_dwork + L.face_off, L.nface);
+        }
+        for (int s = 0; s < ns; ++s) {
+          const bt::SysStep& d = bt->host_steps[off + s];
+          if (d.active == 2 && !d.cplx)
             nonlocal_add_fp64(bt->hams[s], d.X, d.ldx, d.Z, d.ldz, d.ncol, d.alpha);
         }
         for (int c = 0; c < bt->ncolours; ++c) {
@@ -401,6 +486,8 @@ extern "C" dftfe_status dftfe_batch_destroy(dftfe_batch b) {
     if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   if (b->capture_stream) cudaStreamDestroy(b->capture_stream);
   for (auto& kv : b->tail_ws) kv.second.release();
+  b->sf_desc.release();
+  b->mixed_desc.release();
   delete b;
   ABI_END
 }

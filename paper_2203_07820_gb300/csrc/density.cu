@@ -97,35 +97,72 @@ __device__ __forceinline__ double fermi_dirac(double eps, double mu, double kT) 
   return 1.0 / (1.0 + exp(x));
 }
 
-// one thread: bisection on the electron count (increasing in mu), 200 halvings
-__global__ void k_fermi(const double* __restrict__ eps, int nfr, int n_oc, double n_elec, double kT,
-                        double* __restrict__ f, double* __restrict__ mu_out, int* status) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Bisection on the electron count (increasing in mu), at most 200 halvings: one CTA sums the
+// occupations of a halving in parallel (fixed order), and stops once no value lies strictly
+// between the ends (further halvings change neither).  Latency-bound: one thread adding the
+// exponentials one by one took 14.6 ms for 64 states.
+constexpr int kFermiThreads = 256;
+__device__ __forceinline__ double fermi_sum(double v, double* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+#pragma unroll
+  for (int w = 0; w < kFermiThreads / 32; ++w) t += red[w];
+  return t;
+}
+__global__ void __launch_bounds__(kFermiThreads) k_fermi(const double* __restrict__ eps, int nfr, int n_oc,
+                                                         double n_elec, double kT, double* __restrict__ f,
+                                                         double* __restrict__ mu_out, int* status) {
+  __shared__ double red[kFermiThreads / 32], ends[2][kFermiThreads / 32];
   if (!(2.0 * n_oc < n_elec && n_elec < 2.0 * (n_oc + nfr))) {
-    *status = (int)DFTFE_ERR_ARG;
+    if (threadIdx.x == 0) *status = (int)DFTFE_ERR_ARG;
     return;
   }
   double lo = eps[0], hi = eps[0];
-  for (int i = 1; i < nfr; ++i) {
+  for (int i = threadIdx.x; i < nfr; i += kFermiThreads) {
     lo = fmin(lo, eps[i]);
     hi = fmax(hi, eps[i]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    ends[0][threadIdx.x >> 5] = lo;
+    ends[1][threadIdx.x >> 5] = hi;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kFermiThreads / 32; ++w) {
+    lo = fmin(lo, ends[0][w]);
+    hi = fmax(hi, ends[1][w]);
   }
   lo -= 50.0 * kT;
   hi += 50.0 * kT;
   for (int it = 0; it < 200; ++it) {
     const double mid = 0.5 * (lo + hi);
+    if (mid <= lo || mid >= hi) break;        // the same in every thread
     double s = 0.0;
-    for (int i = 0; i < nfr; ++i) s += fermi_dirac(eps[i], mid, kT);
+    for (int i = threadIdx.x; i < nfr; i += kFermiThreads) s += fermi_dirac(eps[i], mid, kT);
+    s = fermi_sum(s, red);
     if (2.0 * (n_oc + s) < n_elec) lo = mid;
     else hi = mid;
   }
   const double mu = 0.5 * (lo + hi);
-  for (int i = 0; i < nfr; ++i) f[i] = fermi_dirac(eps[i], mu, kT);
-  *mu_out = mu;
-  *status = 0;
+  for (int i = threadIdx.x; i < nfr; i += kFermiThreads) f[i] = fermi_dirac(eps[i], mu, kT);
+  if (threadIdx.x == 0) {
+    *mu_out = mu;
+    *status = 0;
+  }
 }
 
 // ---------------------------------------------------------------- density
+// Meshes whose quadrature has p + 1 points per axis or sits on the nodes use the 1D contractions of
+// sumfac.cu; the other rules this dense interpolation.
 // One CTA per cell.  Columns of [Xo | Xfr] are processed 32 at a time: the cell's rows are
 // gathered into shared memory scaled by M^-1/2, each warp interpolates 8 quadrature points
 // at a time (rows of Nq, warp-uniform loads), squares, weights (1 for Psi_o, f - 1 for
@@ -241,7 +278,7 @@ extern "C" dftfe_status dftfe_fermi_level(const double* evals_fr, int nfr, int n
   // two scalars of scratch: allocated per call (the call is outside the pass's hot loop)
   DFTFE_CHECK_CUDA(cudaMallocAsync((void**)&d_mu, sizeof(double) + sizeof(int) * 2, s));
   d_st = (int*)(d_mu + 1);
-  DFTFE_LAUNCH(k_fermi, 1, 32, 0, s, evals_fr, nfr, n_oc, n_elec, kT, f_fr, d_mu, d_st);
+  DFTFE_LAUNCH(k_fermi, 1, kFermiThreads, 0, s, evals_fr, nfr, n_oc, n_elec, kT, f_fr, d_mu, d_st);
   double hmu = 0.0;
   int hst = 0;
   DFTFE_CHECK_CUDA(cudaMemcpyAsync(&hmu, d_mu, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -260,6 +297,11 @@ extern "C" dftfe_status dftfe_density(dftfe_ham h, const double* Xo, int64_t ldo
   DFTFE_REQUIRE(ncol >= 0 && ldo >= ncol && nfr >= 0, "bad sizes");
   DFTFE_REQUIRE(nfr == 0 || (Xfr && f_fr && ldfr >= nfr), "null split-state inputs");
   auto* m = h->mesh;
+  if (sf_applicable(m)) {
+    ProfScope ps(h, "density");
+    sf_density(h, Xo, ldo, ncol, Xfr, ldfr, nfr, f_fr, rho);
+    return DFTFE_OK;
+  }
   static bool attr = false;
   if (!attr) {
     DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_density, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));

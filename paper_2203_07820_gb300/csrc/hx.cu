@@ -1,6 +1,9 @@
 // H~ X application (a4, a5) and the Chebyshev filter (a6).
 //
-// Local part (Sec. 4.3, Eq. celldgemm): Y = ASEMB_FEM{ H~^c X^c }.  One CTA takes one
+// Local part (Sec. 4.3, Eq. celldgemm): Y = ASEMB_FEM{ H~^c X^c }, by the 1D contractions of
+// sumfac.cu where the potential quadrature allows it (p + 1 points per axis, the default, or
+// the nodes), with the recurrence terms fused; the dense cell products here serve the other
+// quadrature rules.  In them one CTA takes one
 // cell and up to 32 columns: it gathers the cell's rows of X into shared memory
 // (each row is a contiguous run of columns, so the gather is coalesced, as in the
 // paper's DoF-major layout), multiplies by the dense cell matrix and adds the result
@@ -44,28 +47,45 @@ __global__ void k_copy_block(const double* __restrict__ src, int64_t lds, double
   dst[i * ldd + j] = src[i * lds + j];
 }
 
-// P[a][col] = h_a * sum_{e in supp a} C~[e] X[node_e][col]; one CTA per (projector, 32 cols).
-__global__ void __launch_bounds__(256) k_nl_coef(const double* __restrict__ X, int64_t ldx, int ncol,
-                                                 const int64_t* __restrict__ prow,
-                                                 const int32_t* __restrict__ pnode,
-                                                 const double* __restrict__ pval,
-                                                 const double* __restrict__ hcoup, double* __restrict__ P) {
+// P[a][col] = h_a * sum_{e in supp a} C~[e] X[node_e][col], the sum split over each projector's
+// support so that a long support (thousands of entries) is not one chain of dependent loads per
+// warp: CTA (a, s) sums range s (warp w every 8th entry, four in flight, lane = column) into
+// part[a S + s]; k_nl_coef_reduce adds the S ranges in order.
+constexpr int kNlSplits64 = 8;
+__global__ void __launch_bounds__(256) k_nl_coef_part(const double* __restrict__ X, int64_t ldx, int ncol,
+                                                      const int64_t* __restrict__ prow,
+                                                      const int32_t* __restrict__ pnode,
+                                                      const double* __restrict__ pval, double* __restrict__ part) {
   __shared__ double red[8][32];
-  const int a = blockIdx.x;
+  const int a = blockIdx.x / kNlSplits64, sidx = blockIdx.x % kNlSplits64;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.y * 32 + lane;
+  const int64_t e0 = prow[a], e1 = prow[a + 1], len = (e1 - e0 + kNlSplits64 - 1) / kNlSplits64;
+  const int64_t s0 = e0 + sidx * len, s1 = min(e1, s0 + len);
   double s = 0.0;
-  if (col < ncol)
-    for (int64_t e = prow[a] + warp; e < prow[a + 1]; e += 8)
-      s = fma(pval[e], X[(int64_t)pnode[e] * ldx + col], s);
+  if (col < ncol) {
+#pragma unroll 4
+    for (int64_t e = s0 + warp; e < s1; e += 8) s = fma(pval[e], X[(int64_t)pnode[e] * ldx + col], s);
+  }
   red[warp][lane] = s;
   __syncthreads();
   if (warp == 0 && col < ncol) {
     double t = 0.0;
 #pragma unroll
     for (int w = 0; w < 8; ++w) t += red[w][lane];
-    P[(int64_t)a * ncol + col] = hcoup[a] * t;
+    part[(int64_t)blockIdx.x * ncol + col] = t;
   }
+}
+
+__global__ void k_nl_coef_reduce(const double* __restrict__ part, const double* __restrict__ hcoup, int nproj,
+                                 int ncol, double* __restrict__ P) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= (int64_t)nproj * ncol) return;
+  const int64_t a = t / ncol;
+  const int col = (int)(t - a * ncol);
+  double s = 0.0;
+  for (int k = 0; k < kNlSplits64; ++k) s += part[(a * kNlSplits64 + k) * ncol + col];
+  P[t] = hcoup[a] * s;
 }
 
 // Z[node][col] += alpha * sum_{t in node's projectors} C~[t] P[proj_t][col]; one warp per node.
@@ -204,7 +224,8 @@ static void local_part_rows(dftfe_ham h, const double* X, int64_t ldx, double* Z
 // Autotuner (no counterpart in the paper, whose cell GEMMs go to a vendor batched GEMM): the
 // first local part of a given column count times every rows-per-CTA shape of the wide
 // kernel (64, 128, ... rows of a cell per CTA, and the heuristic) on the caller's X into a
-// scratch output, twice each (the first run warms up), and keeps the fastest for the ham.
+// scratch output, twice each (the first run warms up), and keeps the fastest for the ham.  The
+// tensor-product form has one launch shape: it is timed as the heuristic.
 static int tuned_rows(dftfe_ham h, const double* X, int64_t ldx, int ncol) {
   auto it = h->tuned_fp64.find(ncol);
   if (it != h->tuned_fp64.end()) return it->second.rows;
@@ -224,10 +245,15 @@ static int tuned_rows(dftfe_ham h, const double* X, int64_t ldx, int ncol) {
   TunedShape best;
   best.best_ms = 1e300;
   try {
-    for (int r = 0; r <= (m->nc + 63) / 64 * 64; r += 64) {
-      local_part_rows(h, X, ldx, Zs, ncol, ncol, 1.0, r);
+    const bool sf = sf_applicable(m);
+    auto run = [&](int r) {
+      if (sf) sf_local64(h, X, ldx, nullptr, 0, Zs, ncol, ncol, 1.0, 0.0, 0.0);
+      else local_part_rows(h, X, ldx, Zs, ncol, ncol, 1.0, r);
+    };
+    for (int r = 0; r <= (sf ? 0 : (m->nc + 63) / 64 * 64); r += 64) {
+      run(r);
       DFTFE_CHECK_CUDA(cudaEventRecord(ev.e[0], h->stream));
-      local_part_rows(h, X, ldx, Zs, ncol, ncol, 1.0, r);
+      run(r);
       DFTFE_CHECK_CUDA(cudaEventRecord(ev.e[1], h->stream));
       DFTFE_CHECK_CUDA(cudaEventSynchronize(ev.e[1]));
       float ms = 0.f;
@@ -250,15 +276,24 @@ static int tuned_rows(dftfe_ham h, const double* X, int64_t ldx, int ncol) {
 void local_part_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Z, int64_t ldz, int ncol,
                      double alpha) {
   const int rows = h->autotune && ncol > 4 ? tuned_rows(h, X, ldx, ncol) : 0;
-  local_part_rows(h, X, ldx, Z, ldz, ncol, alpha, rows);
+  if (sf_applicable(h->mesh)) sf_local64(h, X, ldx, Z, ldz, Z, ldz, ncol, alpha, 0.0, 1.0);
+  else local_part_rows(h, X, ldx, Z, ldz, ncol, alpha, rows);
+}
+
+// P = h (C~^T X)
+static const double* nl_coef64(dftfe_ham h, const double* X, int64_t ldx, int ncol) {
+  double* P = (double*)ws_get(h, "nl_coef", sizeof(double) * h->nproj * (size_t)ncol);
+  double* part = (double*)ws_get(h, "nl_coef_part", sizeof(double) * h->nproj * (size_t)kNlSplits64 * ncol);
+  dim3 grid((unsigned)(h->nproj * kNlSplits64), (unsigned)((ncol + 31) / 32));
+  DFTFE_LAUNCH(k_nl_coef_part, grid, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, h->d_pval, part);
+  DFTFE_LAUNCH(k_nl_coef_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, h->stream, part, h->d_h, h->nproj, ncol, P);
+  return P;
 }
 
 // Z += alpha H~_nl X (FP64), nothing without projectors
 void nonlocal_add_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Z, int64_t ldz, int ncol, double alpha) {
   if (h->nproj <= 0) return;
-  double* P = (double*)ws_get(h, "nl_coef", sizeof(double) * h->nproj * (size_t)ncol);
-  dim3 g1((unsigned)h->nproj, (unsigned)((ncol + 31) / 32));
-  DFTFE_LAUNCH(k_nl_coef, g1, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, h->d_pval, h->d_h, P);
+  const double* P = nl_coef64(h, X, ldx, ncol);
   dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
   DFTFE_LAUNCH(k_nl_add, g2, 256, 0, h->stream, Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P,
                h->nsup, alpha);
@@ -269,6 +304,13 @@ void apply_combo(dftfe_ham h, const double* X, int64_t ldx, const double* Xprev,
   if (!loc(h)->has_potential) throw Error(DFTFE_ERR_STATE, "set the potential before applying H");
   auto* m = h->mesh;
   if (ncol <= 0) return;
+  if (sf_applicable(m)) {
+    // the recurrence terms ride in the cell and face kernels; the projectors are added on top
+    if (h->autotune && ncol > 4) tuned_rows(h, X, ldx, ncol);
+    sf_local64(h, X, ldx, Xprev, ldp, Z, ldz, ncol, alpha, s1, s2);
+    nonlocal_add_fp64(h, X, ldx, Z, ldz, ncol, alpha);
+    return;
+  }
   set_smem_attrs();
   DFTFE_LAUNCH(k_axpby_init, nblk(m->M * ncol), 256, 0, h->stream, Z, ldz, X, ldx, Xprev, ldp, m->M,
                ncol, s1, s2);
@@ -281,9 +323,7 @@ void apply_nonlocal_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Y, i
   DFTFE_LAUNCH(k_axpby_init, nblk(m->M * ncol), 256, 0, h->stream, Y, ldy, X, ldx, nullptr, 0, m->M, ncol, 0.0,
                0.0);
   if (h->nproj > 0) {
-    double* P = (double*)ws_get(h, "nl_coef", sizeof(double) * h->nproj * (size_t)ncol);
-    dim3 g1((unsigned)h->nproj, (unsigned)((ncol + 31) / 32));
-    DFTFE_LAUNCH(k_nl_coef, g1, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, h->d_pval, h->d_h, P);
+    const double* P = nl_coef64(h, X, ldx, ncol);
     dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
     DFTFE_LAUNCH(k_nl_add, g2, 256, 0, h->stream, Y, ldy, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P,
                  h->nsup, 1.0);

@@ -874,6 +874,27 @@ static MixedShape tune_cell_tf32p(cudaStream_t s, int sm, const mp::Item& one, c
   return best;
 }
 
+// The tensor-product form has one launch shape; its time (one launch, after an untimed one) is
+// recorded as both the best and the default.
+static MixedShape time_sf32(cudaStream_t s, const std::function<void()>& run) {
+  struct Ev {
+    cudaEvent_t e[2] = {nullptr, nullptr};
+    ~Ev() { for (auto x : e) if (x) cudaEventDestroy(x); }
+  } ev;
+  for (auto& x : ev.e) DFTFE_CHECK_CUDA(cudaEventCreate(&x));
+  run();
+  DFTFE_CHECK_CUDA(cudaEventRecord(ev.e[0], s));
+  run();
+  DFTFE_CHECK_CUDA(cudaEventRecord(ev.e[1], s));
+  DFTFE_CHECK_CUDA(cudaEventSynchronize(ev.e[1]));
+  float ms = 0.f;
+  DFTFE_CHECK_CUDA(cudaEventElapsedTime(&ms, ev.e[0], ev.e[1]));
+  MixedShape r;
+  r.atmem = 0;
+  r.best_ms = r.default_ms = ms;
+  return r;
+}
+
 static void set_tf32p_attrs() {
   DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_cell_tf32p<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)mp::smem_bytes<true, false>()));
@@ -922,6 +943,7 @@ __global__ void __launch_bounds__(256) k_nl_coef32_part(const float* __restrict_
   const int64_t s0 = e0 + sidx * len, s1 = min(e1, s0 + len);
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c0 < ncol) {
+#pragma unroll 4
     for (int64_t e = s0 + warp; e < s1; e += 8) {
       const float w = (float)pval[e];
       const float4 x = __ldg(reinterpret_cast<const float4*>(X + (int64_t)pnode[e] * ldx + c0));
@@ -953,8 +975,50 @@ __global__ void k_nl_coef32_reduce(const float* __restrict__ part, const double*
   P[(int64_t)a * ldP + col] = (float)hcoup[a] * s;
 }
 
+// Z[node] += alpha sum_t w_t P[a_t] on the support nodes (the tensor-product form, whose cell and
+// face kernels write Z without the projectors): one warp per node, four columns per lane
+__global__ void __launch_bounds__(256) k_nl_add32(float* __restrict__ Z, int64_t ldz, int ncol,
+                                                  const int32_t* __restrict__ snode, const int64_t* __restrict__ srow,
+                                                  const int32_t* __restrict__ sproj, const double* __restrict__ sval,
+                                                  const float* __restrict__ P, int ldP, int64_t nsup, float alpha) {
+  const int64_t s = blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int c = blockIdx.y * 128 + 4 * (threadIdx.x & 31);
+  if (s >= nsup || c >= ncol) return;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int64_t t = srow[s]; t < srow[s + 1]; ++t) {
+    const float w = (float)sval[t];
+    const float4 pv = *reinterpret_cast<const float4*>(P + (int64_t)sproj[t] * ldP + c);   // ldP % 4 == 0
+    acc.x = fmaf(w, pv.x, acc.x); acc.y = fmaf(w, pv.y, acc.y);
+    acc.z = fmaf(w, pv.z, acc.z); acc.w = fmaf(w, pv.w, acc.w);
+  }
+  float* z = Z + (int64_t)snode[s] * ldz + c;
+  if (c + 3 < ncol) {
+    float4 v = *reinterpret_cast<float4*>(z);
+    v.x = fmaf(alpha, acc.x, v.x); v.y = fmaf(alpha, acc.y, v.y);
+    v.z = fmaf(alpha, acc.z, v.z); v.w = fmaf(alpha, acc.w, v.w);
+    *reinterpret_cast<float4*>(z) = v;
+  } else {
+    const float a[4] = {acc.x, acc.y, acc.z, acc.w};
+    for (int j = 0; c + j < ncol; ++j) z[j] = fmaf(alpha, a[j], z[j]);
+  }
+}
 
 static unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
+
+static void nl_add32(dftfe_ham h, cudaStream_t s, float* Z, int64_t ldz, int ncol, const float* P, int ldP,
+                     float alpha) {
+  dim3 grid((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 127) / 128));
+  DFTFE_LAUNCH(k_nl_add32, grid, 256, 0, s, Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P, ldP,
+               h->nsup, alpha);
+}
+
+// the split-precision form of this mesh: the FP32 tensor-product kernels, whose products carry
+// 24 bits where the 3-term splits carry 21, or (other quadrature rules, BF16x3) split dense products
+static bool use_sf32(dftfe_ham h, bool tf32) { return tf32 && sf_applicable(h->mesh); }
+static void check_mixed_degree(dftfe_ham h) {
+  if (h->mesh->nc > 128 * mx::kMaxMTiles)
+    throw Error(DFTFE_ERR_ARG, "mixed precision supports at most 512 nodes per cell (p <= 7)");
+}
 
 static size_t mixed_smem() {
   return 1024 + (size_t)mx::kStagesA * mx::kStageBytes + (size_t)mx::kStagesB * mx::kStageBytes + mx::kPatchBytes +
@@ -1086,11 +1150,7 @@ static void apply_combo_mixed(dftfe_ham h, bool tf32, const uint8_t* A, int nkc,
     const double k2 = h->kvec[0] * h->kvec[0] + h->kvec[1] * h->kvec[1] + h->kvec[2] * h->kvec[2];
     s1 += (float)(0.5 * (double)alpha * k2);
   }
-  const int32_t *nptr, *nslot;
-  node_slots(h, &nptr, &nslot);
-  float* Yc = (float*)ws_get(h, "mx_yc", sizeof(float) * (size_t)m->Nc * m->nc * 128);
-  const size_t sh = mixed_smem();
-  const unsigned grid = (unsigned)std::min<int64_t>(m->Nc, h->sm_count);
+  const bool sf = use_sf32(h, tf32);
   // nonlocal coefficients P = h (C~^T X) first: the assembly adds C~ P with the cell sums
   float* P = nullptr;
   const int ldP = (ncol + 3) / 4 * 4;
@@ -1102,6 +1162,30 @@ static void apply_combo_mixed(dftfe_ham h, bool tf32, const uint8_t* A, int nkc,
     DFTFE_LAUNCH(k_nl_coef32_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, h->stream, Pp, h->d_h, h->nproj,
                  ncol, P, ldP);
   }
+  if (sf) {
+    const float* v = sf_potential32(h);
+    float* face = (float*)ws_get(h, "sf_face", sizeof(float) * sf_face_elems(m, std::min(ncol, kSfCols)));
+    for (int c0 = 0; c0 < ncol; c0 += kSfCols) {
+      const int nb = std::min(kSfCols, ncol - c0);
+      const sf::Item<float> one = sf_item32(h, v, face, X + c0, ldx, Xp ? Xp + c0 : nullptr, ldp, Z + c0, ldz, nb, alpha,
+                                            s1, s2);
+      auto run = [&]() { sf_launch32(h->stream, h->sm_count, m, kpoint, one, nullptr, nullptr, sf_cell_work32(m, nb), nullptr, m->Nc); };
+      if (h->autotune && !h->tuned_mixed_done && !capturing(h->stream)) {
+        h->tuned_mixed = time_sf32(h->stream, run);
+        h->tuned_mixed_done = true;
+      }
+      ProfScope ps(h, "cell_gemm_tf32x3");
+      run();
+    }
+    if (P) nl_add32(h, h->stream, Z, ldz, ncol, P, ldP, alpha);
+    if (kpoint) kpoint_add32(h, X, ldx, Z, ldz, ncol / 2, alpha, false);
+    return;
+  }
+  const int32_t *nptr, *nslot;
+  node_slots(h, &nptr, &nslot);
+  float* Yc = (float*)ws_get(h, "mx_yc", sizeof(float) * (size_t)m->Nc * m->nc * 128);
+  const size_t sh = mixed_smem();
+  const unsigned grid = (unsigned)std::min<int64_t>(m->Nc, h->sm_count);
   for (int col0 = 0; col0 < ncol; col0 += 128) {
     {
       ProfScope ps(h, tf32 ? "cell_gemm_tf32x3" : "cell_gemm_bf16x3");
@@ -1138,8 +1222,9 @@ void chebyshev_filter_mixed(dftfe_ham h, double* X, int64_t ld, int ncol, int de
     DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_cell_mixed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mixed_smem()));
     g_mixed_attr = true;
   }
-  int nkc, nmt;
-  const uint8_t* A = mixed_tiles(h, tf32, &nkc, &nmt);
+  int nkc = 0, nmt = 0;
+  check_mixed_degree(h);
+  const uint8_t* A = use_sf32(h, tf32) ? nullptr : mixed_tiles(h, tf32, &nkc, &nmt);
   const int64_t ld32 = (ncol + 31) / 32 * 32;
   float* buf[3];
   buf[0] = (float*)ws_get(h, "mx_v0", sizeof(float) * m->M * (size_t)ld32);
@@ -1205,6 +1290,19 @@ struct MixedRoundPlan {
     float* Yc = nullptr;
     float* buf[3] = {nullptr, nullptr, nullptr};
     int64_t ld32 = 0;
+    bool sf = false;                  // tensor-product form: its scaled potential and face buffer
+    const float* v = nullptr;
+    float* face = nullptr;
+  };
+  // one launch of the tensor-product kernels: the systems of one degree, quadrature rule and kind
+  // (Gamma or k-point) still filtering at step k
+  struct SfLaunch {
+    int k;
+    const dftfe_mesh_s* mesh;
+    bool kpoint;
+    size_t item_off, cell_off, face_off;
+    int nitems;
+    int64_t ncell, nface;
   };
   struct StepSys {
     int cur, prev, out;
@@ -1220,6 +1318,8 @@ struct MixedRoundPlan {
   std::vector<Sys> sy;
   std::vector<std::vector<StepSys>> steps;
   std::vector<CellLaunch> launches;
+  std::vector<SfLaunch> sf_launches;
+  size_t sf_base = 0;                      // element offset of the round's tensor-product items
   int maxdeg = 0, ntiles = 0;
   size_t item_base = 0, work_base = 0;     // element offsets of the round in the uploads
 };
@@ -1246,15 +1346,23 @@ static void plan_mixed_round(MixedRoundPlan& R, std::vector<mp::Item>& items, st
     dftfe_ham h = b.h;
     auto* m = h->mesh;
     Sys& y = sy[s];
-    y.A = mixed_tiles(h, true, &y.nkc, &y.nmt);
-    node_slots(h, &y.nptr, &y.nslot);
-    y.Yc = (float*)ws_get(h, "mx_yc", sizeof(float) * (size_t)m->Nc * m->nc * 128);
+    check_mixed_degree(h);
+    y.sf = use_sf32(h, true);
+    if (y.sf) {
+      y.v = sf_potential32(h);
+      // the widest block first: every round's items point into the one face buffer
+      y.face = (float*)ws_get(h, "sf_face", sizeof(float) * sf_face_elems(m, b.ncol));
+    } else {
+      y.A = mixed_tiles(h, true, &y.nkc, &y.nmt);
+      node_slots(h, &y.nptr, &y.nslot);
+      y.Yc = (float*)ws_get(h, "mx_yc", sizeof(float) * (size_t)m->Nc * m->nc * 128);
+    }
     y.ld32 = (b.ncol + 31) / 32 * 32;
     y.buf[0] = (float*)ws_get(h, "mx_v0", sizeof(float) * m->M * (size_t)y.ld32);
     y.buf[1] = (float*)ws_get(h, "mx_v1", sizeof(float) * m->M * (size_t)y.ld32);
     y.buf[2] = (float*)ws_get(h, "mx_v2", sizeof(float) * m->M * (size_t)y.ld32);
     maxdeg = std::max(maxdeg, b.degree);
-    ntiles = std::max(ntiles, (b.ncol + 127) / 128);
+    if (!y.sf) ntiles = std::max(ntiles, (b.ncol + 127) / 128);
   }
   // buffer rotation and recurrence coefficients of every system and step, as the single filter
   // forms them
@@ -1306,14 +1414,15 @@ static void plan_mixed_round(MixedRoundPlan& R, std::vector<mp::Item>& items, st
   launches.clear();
   std::vector<int> ncs;
   for (int s = 0; s < ns; ++s)
-    if (!steps[s].empty() && std::find(ncs.begin(), ncs.end(), blk[s].h->mesh->nc) == ncs.end())
+    if (!steps[s].empty() && !sy[s].sf && std::find(ncs.begin(), ncs.end(), blk[s].h->mesh->nc) == ncs.end())
       ncs.push_back(blk[s].h->mesh->nc);
   for (int k = 1; k <= maxdeg; ++k)
     for (int t = 0; t < ntiles; ++t)
       for (int nc : ncs) {
         std::vector<int> act;
         for (int s = 0; s < ns; ++s)
-          if ((int)steps[s].size() >= k && blk[s].h->mesh->nc == nc && blk[s].ncol > 128 * t) act.push_back(s);
+          if ((int)steps[s].size() >= k && !sy[s].sf && blk[s].h->mesh->nc == nc && blk[s].ncol > 128 * t)
+            act.push_back(s);
         if (act.empty()) continue;
         CellLaunch L{k, t, nc, sy[act[0]].nkc, sy[act[0]].nmt, items.size() - R.item_base, 0, 0, 0,
                      (int)act.size(), MixedShape{}};
@@ -1346,8 +1455,51 @@ static void plan_mixed_round(MixedRoundPlan& R, std::vector<mp::Item>& items, st
       }
 }
 
+// tensor-product launches of a round, after plan_mixed_round has formed its steps
+static void plan_sf_round(MixedRoundPlan& R, std::vector<int2>& work, std::vector<sf::Item<float>>& sf_items) {
+  const int ns = (int)R.blk.size();
+  std::map<std::vector<int>, MixedRoundPlan::SfLaunch> lists;      // by the systems they cover
+  for (int k = 1; k <= R.maxdeg; ++k) {
+    std::map<std::vector<int>, std::vector<int>> groups;
+    for (int s = 0; s < ns; ++s)
+      if (R.sy[s].sf && (int)R.steps[s].size() >= k) {
+        const auto* m = R.blk[s].h->mesh;
+        groups[{m->n1, m->vquad, R.blk[s].kpoint ? 1 : 0}].push_back(s);
+      }
+    for (auto& g : groups) {
+      const std::vector<int>& act = g.second;
+      auto it = lists.find(act);
+      if (it == lists.end()) {
+        MixedRoundPlan::SfLaunch L{0, R.blk[act[0]].h->mesh, R.blk[act[0]].kpoint, 0, work.size() - R.work_base, 0,
+                                   (int)act.size(), 0, 0};
+        for (size_t q = 0; q < act.size(); ++q) {
+          const int64_t n = sf_cell_work32(R.blk[act[q]].h->mesh, R.blk[act[q]].ncol);
+          for (int64_t t = 0; t < n; ++t) work.push_back(make_int2((int)q, (int)t));
+        }
+        L.face_off = work.size() - R.work_base;
+        L.ncell = (int64_t)(L.face_off - L.cell_off);
+        for (size_t q = 0; q < act.size(); ++q)
+          for (int64_t t = 0; t < R.blk[act[q]].h->mesh->Nc; ++t) work.push_back(make_int2((int)q, (int)t));
+        L.nface = (int64_t)(work.size() - R.work_base - L.face_off);
+        it = lists.emplace(act, L).first;
+      }
+      MixedRoundPlan::SfLaunch L = it->second;
+      L.k = k;
+      L.item_off = sf_items.size() - R.sf_base;
+      for (int s : act) {
+        const auto& y = R.sy[s];
+        const auto& st = R.steps[s][k - 1];
+        sf_items.push_back(sf_item32(R.blk[s].h, y.v, y.face, y.buf[st.cur], y.ld32,
+                                     st.prev >= 0 ? y.buf[st.prev] : nullptr, y.ld32, y.buf[st.out], y.ld32,
+                                     R.blk[s].ncol, st.alpha, st.s1, st.s2));
+      }
+      R.sf_launches.push_back(L);
+    }
+  }
+}
+
 static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, int* err, const mp::Item* d_items,
-                                const int2* d_work) {
+                                const int2* d_work, const sf::Item<float>* d_sf) {
   using StepSys = MixedRoundPlan::StepSys;
   using CellLaunch = MixedRoundPlan::CellLaunch;
   const std::vector<MixedBlock>& blk = R.blk;
@@ -1365,7 +1517,7 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
       DFTFE_LAUNCH(k_to_f32, nblk(m->M * blk[s].ncol), 256, 0, stream, blk[s].X, blk[s].ld, sy[s].buf[0], sy[s].ld32,
                    m->M, blk[s].ncol);
     }
-  size_t li = 0;
+  size_t li = 0, lsf = 0;
   for (int k = 1; k <= maxdeg; ++k) {
     // nonlocal coefficients P = h (C~^T X) of the Gamma-point systems with projectors
     std::vector<float*> P(ns, nullptr);
@@ -1385,6 +1537,17 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
       DFTFE_LAUNCH(k_nl_coef32_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, stream, Pp, h->d_h, h->nproj, ncol,
                    P[s], ldP[s]);
     }
+    for (; lsf < R.sf_launches.size() && R.sf_launches[lsf].k == k; ++lsf) {
+      const auto& L = R.sf_launches[lsf];
+      ProfScope ps(blk[0].h, "batch_cell_tf32x3");
+      sf_launch32(stream, sm, L.mesh, L.kpoint, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
+                  d_work + R.work_base + L.cell_off, L.ncell, d_work + R.work_base + L.face_off, L.nface);
+    }
+    for (int s = 0; s < ns; ++s)
+      if (sy[s].sf && P[s]) {
+        const StepSys& st = steps[s][k - 1];
+        nl_add32(blk[s].h, stream, sy[s].buf[st.out], sy[s].ld32, blk[s].ncol, P[s], ldP[s], st.alpha);
+      }
     for (int t = 0; t < ntiles; ++t) {
       for (; li < launches.size() && launches[li].k == k && launches[li].tile == t; ++li) {
         const CellLaunch& L = launches[li];
@@ -1395,7 +1558,7 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
                           L.nmt, err, L.shape);
       }
       for (int s = 0; s < ns; ++s) {
-        if ((int)steps[s].size() < k || blk[s].ncol <= 128 * t) continue;
+        if ((int)steps[s].size() < k || sy[s].sf || blk[s].ncol <= 128 * t) continue;
         dftfe_ham h = blk[s].h;
         auto* m = h->mesh;
         const StepSys& st = steps[s][k - 1];
@@ -1411,7 +1574,8 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
     for (int s = 0; s < ns; ++s) {
       if ((int)steps[s].size() < k || !blk[s].kpoint) continue;
       const StepSys& st = steps[s][k - 1];
-      kpoint_add32(blk[s].h, sy[s].buf[st.cur], sy[s].ld32, sy[s].buf[st.out], sy[s].ld32, blk[s].ncol / 2, st.alpha);
+      kpoint_add32(blk[s].h, sy[s].buf[st.cur], sy[s].ld32, sy[s].buf[st.out], sy[s].ld32, blk[s].ncol / 2, st.alpha,
+                   !sy[s].sf);
     }
   }
   for (int s = 0; s < ns; ++s)
@@ -1433,28 +1597,50 @@ std::function<void()> plan_mixed_batch(const std::vector<std::vector<MixedBlock>
   auto plans = std::make_shared<std::vector<MixedRoundPlan>>(rounds.size());
   std::vector<mp::Item> items;
   std::vector<int2> work;
+  std::vector<sf::Item<float>> sf_items;
+  // buffers that several rounds point into, at the size of a system's widest block
+  for (const auto& r : rounds)
+    for (const MixedBlock& b : r)
+      if (b.degree > 0 && b.ncol > 0 && use_sf32(b.h, true))
+        ws_get(b.h, "sf_face", sizeof(float) * sf_face_elems(b.h->mesh, b.ncol));
   for (size_t j = 0; j < rounds.size(); ++j) {
     MixedRoundPlan& R = (*plans)[j];
     R.blk = rounds[j];
     R.item_base = items.size();
     R.work_base = work.size();
+    R.sf_base = sf_items.size();
     plan_mixed_round(R, items, work);
+    plan_sf_round(R, work, sf_items);
   }
   const size_t ib = items.size() * sizeof(mp::Item), wb = work.size() * sizeof(int2);
-  const size_t woff = (ib + 255) / 256 * 256;
-  host_desc.resize(std::max<size_t>(woff + wb, 1));
+  const size_t sb = sf_items.size() * sizeof(sf::Item<float>);
+  const size_t woff = (ib + 255) / 256 * 256, soff = (woff + wb + 255) / 256 * 256;
+  host_desc.resize(std::max<size_t>(soff + sb, 1));
   if (ib) std::memcpy(host_desc.data(), items.data(), ib);
   if (wb) std::memcpy(host_desc.data() + woff, work.data(), wb);
+  if (sb) std::memcpy(host_desc.data() + soff, sf_items.data(), sb);
+  if (host_desc.size() > desc.bytes) DFTFE_CHECK_CUDA(cudaStreamSynchronize(stream));
   uint8_t* ddesc = (uint8_t*)desc.get(host_desc.size());
   // from pageable memory: the call returns once the data is staged, so the host copy may be
   // rewritten by the next pass
   DFTFE_CHECK_CUDA(cudaMemcpyAsync(ddesc, host_desc.data(), host_desc.size(), cudaMemcpyHostToDevice, stream));
   const mp::Item* d_items = reinterpret_cast<const mp::Item*>(ddesc);
   const int2* d_work = reinterpret_cast<const int2*>(ddesc + woff);
+  const sf::Item<float>* d_sf = reinterpret_cast<const sf::Item<float>*>(ddesc + soff);
   // launch shapes: the tuned shape of each distinct launch (FE degree, systems, work items),
   // timed on its first appearance when the batch tunes, else the default shape
   if (tuned) {
     const int sm = rounds.empty() || rounds[0].empty() ? 1 : rounds[0][0].h->sm_count;
+    for (MixedRoundPlan& R : *plans)
+      for (auto& L : R.sf_launches) {
+        const std::string key = std::to_string(L.mesh->nc) + "/" + std::to_string(L.ncell) + "/" +
+                                std::to_string(L.nitems) + (L.kpoint ? "/sf_z" : "/sf");
+        if (tuned->count(key) || capturing(stream)) continue;
+        (*tuned)[key] = time_sf32(stream, [&]() {
+          sf_launch32(stream, sm, L.mesh, L.kpoint, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
+                      d_work + R.work_base + L.cell_off, L.ncell, d_work + R.work_base + L.face_off, L.nface);
+        });
+      }
     for (MixedRoundPlan& R : *plans)
       for (auto& L : R.launches) {
         // key: FE degree (nodes per cell), work items, systems and distinct cell-matrix planes
@@ -1476,8 +1662,8 @@ std::function<void()> plan_mixed_batch(const std::vector<std::vector<MixedBlock>
         L.shape = it->second;
       }
   }
-  return [plans, stream, err, d_items, d_work]() {
-    for (const MixedRoundPlan& R : *plans) enqueue_mixed_round(R, stream, err, d_items, d_work);
+  return [plans, stream, err, d_items, d_work, d_sf]() {
+    for (const MixedRoundPlan& R : *plans) enqueue_mixed_round(R, stream, err, d_items, d_work, d_sf);
   };
 }
 
@@ -1489,8 +1675,9 @@ void apply_mixed(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t l
     DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_cell_mixed<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mixed_smem()));
     g_mixed_attr = true;
   }
-  int nkc, nmt;
-  const uint8_t* A = mixed_tiles(h, tf32, &nkc, &nmt);
+  int nkc = 0, nmt = 0;
+  check_mixed_degree(h);
+  const uint8_t* A = use_sf32(h, tf32) ? nullptr : mixed_tiles(h, tf32, &nkc, &nmt);
   const int64_t ld32 = (ncol + 31) / 32 * 32;
   float* x32 = (float*)ws_get(h, "mx_v0", sizeof(float) * m->M * (size_t)ld32);
   float* y32 = (float*)ws_get(h, "mx_v1", sizeof(float) * m->M * (size_t)ld32);

@@ -12,6 +12,7 @@
 #include <functional>
 
 #include "../../include/dftfe_gb300.h"
+#include "sumfac.h"
 
 namespace dftfe {
 
@@ -147,16 +148,17 @@ struct dftfe_ham_s {
   int32_t* d_node_ptr = nullptr;   // node -> (cell, local row) slots, CSR (built on first mixed use)
   int32_t* d_node_slot = nullptr;
   // a2: cell matrices
-  double* d_K = nullptr;           // nc x nc shared stiffness
-  double* d_P = nullptr;           // Msym x nq packed basis products (Eq. gemmLoc)
-  int32_t* d_pairs = nullptr;      // Msym x 2 (j <= k)
-  double* d_wq = nullptr;          // nq quadrature weights * detJ
+  double* d_celltab = nullptr;     // 1D tables the cell matrices are formed from (sf_init)
   double* d_Nq = nullptr;          // nq x nc basis values at the quadrature points
   double* d_Hc = nullptr;          // Nc x nc x nc FP64
+  // reference quadrature weights, and the cells' potential scaled by them (sumfac.cu)
+  double* d_sfw = nullptr;         // nq
+  double* d_sfv = nullptr;         // Nc x nq
   bool has_potential = false;
   int64_t potential_version = 0;   // bumped by every set_potential
   int64_t mixed_version[2] = {-1, -1};  // potential version of the split tiles (bf16, tf32)
   int64_t df_version = -1;              // potential version of the float-pair cell matrices
+  int64_t sf32_version = -1;            // potential version of the FP32 scaled potential
   int64_t slices_version = -1;          // potential version of the digit rows (exact slices)
   // a3: nonlocal (CSR by projector and by node)
   int nproj = 0;
@@ -248,6 +250,37 @@ void copy_block(cudaStream_t s, const double* src, int64_t lds, double* dst, int
                 int64_t rows, int ncol);
 void zero_block(cudaStream_t s, double* dst, int64_t ldd, int64_t rows, int ncol);
 
+// sumfac.cu: H~_loc X by 1D contractions (meshes whose potential quadrature has p + 1 points per
+// axis or sits on the nodes)
+bool sf_applicable(const dftfe_mesh_s* m);
+void sf_init(dftfe_ham h);                                    // tables of a ham that owns its operator
+void sf_set_potential(dftfe_ham h, const double* v_quad);
+constexpr int kSfCols = 128;                                  // columns per face buffer of a single system
+// Z = s1 X + s2 Xp + alpha H~_loc X in FP64 (Xp may be null or Z)
+void sf_local64(dftfe_ham h, const double* X, int64_t ldx, const double* Xp, int64_t ldp, double* Z, int64_t ldz,
+                int ncol, double alpha, double s1, double s2);
+// batched form: items of meshes of one degree and quadrature rule, work lists of (item, CTA) for
+// the cell kernel (sf_cell_work64 CTAs per item) and (item, cell) for the faces
+size_t sf_face_elems(const dftfe_mesh_s* m, int ncol);
+int64_t sf_cell_work64(const dftfe_mesh_s* m, int ncol);
+sf::Item<double> sf_item64(dftfe_ham h, double* face, const double* X, int64_t ldx, const double* Xp, int64_t ldp,
+                           double* Z, int64_t ldz, int ncol, double alpha, double s1, double s2);
+void sf_launch64(cudaStream_t s, int sm, const dftfe_mesh_s* m, const sf::Item<double>& one, const sf::Item<double>* items,
+                 const int2* cell_work, int64_t ncell_work, const int2* face_work, int64_t nface_work);
+
+// FP32 form (the split-precision filter): rows of every buffer 16-byte aligned, kpoint: complex
+// columns with the k.grad term of the ham's k-point
+const float* sf_potential32(dftfe_ham h);
+sf::Item<float> sf_item32(dftfe_ham h, const float* v, float* face, const float* X, int64_t ldx, const float* Xp,
+                          int64_t ldp, float* Z, int64_t ldz, int ncol, double alpha, double s1, double s2);
+int64_t sf_cell_work32(const dftfe_mesh_s* m, int ncol);
+void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, const sf::Item<float>& one,
+                 const sf::Item<float>* items, const int2* cell_work, int64_t ncell_work, const int2* face_work,
+                 int64_t nface_work);
+
+void sf_density(dftfe_ham h, const double* Xo, int64_t ldo, int ncol, const double* Xfr, int64_t ldf, int nfr,
+                const double* f_fr, double* rho);
+
 // hx_mixed.cu
 // ext_err: a device flag the caller zeroes and reads (a bounded wait timed out); NULL makes
 // the call zero and read its own (and synchronise)
@@ -285,7 +318,9 @@ bool apply_slices(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t 
 void apply_w(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, bool with_nl = true);
 // kpoint.cu: Z += alpha (-i k.grad X + H~_nl^k X) on FP32 complex blocks given by their real
 // views (ld in floats, ncolz complex columns); 1/2|k|^2 is the caller's
-void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ldz, int ncolz, float alpha);
+// (kin = false: the nonlocal term alone)
+void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ldz, int ncolz, float alpha,
+                  bool kin = true);
 // hx.cu: Y = H~_nl X (Y overwritten; zero when there are no projectors), FP64
 void apply_nonlocal_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol);
 

@@ -425,12 +425,12 @@ void apply_combo_z(dftfe_ham h, const double* X, int64_t ldx, const double* Xp, 
   local_part_fp64(h, X, 2 * ldx, Z, 2 * ldz, 2 * ncol, alpha);
 }
 
-void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ldz, int ncolz, float alpha) {
+void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ldz, int ncolz, float alpha, bool kin) {
   require_kpoint(h);
   auto* m = h->mesh;
   if (ncolz <= 0) return;
   const int p = m->p;
-  {
+  if (kin) {
     ProfScope ps(h, "kin_k32");
     const size_t sh = sizeof(float) * 3 * p * (2 * p + 1);
     // 8 nodes per CTA, 64 complex columns per blockIdx.y; the complex row strides ldx / 2 and

@@ -4,10 +4,9 @@
 //    cell -> global map and the lumped diagonal mass M (text after Eq. hep).  On a
 //    uniform periodic mesh M = M1x (x) M1y (x) M1z with M1 the 1D lumped mass, which
 //    is how the device builds it.
-// a2 (Sec. 4.2, Eq. quadLocal / Eq. gemmLoc): V^c for all cells by one packed-symmetric
-//    GEMM K^{eff,loc} = P V with P_{I,q} = N_j(x_q) N_k(x_q) (j <= k) and
-//    V_{q,c} = w_q detJ V(x_q^c); the GLL stiffness K^c = 1/2 int grad N . grad N is
-//    shared by all cells; H~^c = D_c^-1/2 (K^c + V^c) D_c^-1/2 (Eq. hep, Eq. celldgemm).
+// a2 (Sec. 4.2, Eq. quadLocal): H~^c = D_c^-1/2 (K^c + V^c) D_c^-1/2 (Eq. hep, Eq. celldgemm),
+//    V^c one axis at a time from the tensor-product quadrature, the GLL stiffness K^c =
+//    1/2 int grad N . grad N as its Kronecker terms.
 // a3 (Eq. nonlocalHamDiscrete, Alg. 4): C_ja = M_jj chi_a(x_j) (GLL collocation), stored
 //    as C~ = M^1/2 chi in CSR by projector and by node.
 #include "internal.h"
@@ -108,79 +107,88 @@ __global__ void k_mass(double* mass, double* minvsqrt, const double* m1x, const 
   minvsqrt[j] = 1.0 / sqrt(m);
 }
 
-// P[I*nq + q] = N_j(x_q) N_k(x_q), (j, k) = pairs[I], tensor-product basis values.
-__global__ void k_products(double* P, const int32_t* pairs, const double* Lq, int64_t Msym,
-                           int nq1, int n1) {
-  const int nq = nq1 * nq1 * nq1;
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= Msym * nq) return;
-  int64_t I = t / nq;
-  int q = (int)(t % nq);
-  int j = pairs[2 * I], k = pairs[2 * I + 1];
-  int qa = q % nq1, qb = (q / nq1) % nq1, qc = q / (nq1 * nq1);
-  int ja = j % n1, jb = (j / n1) % n1, jc = j / (n1 * n1);
-  int ka = k % n1, kb = (k / n1) % n1, kc = k / (n1 * n1);
-  double Nj = Lq[qa * n1 + ja] * Lq[qb * n1 + jb] * Lq[qc * n1 + jc];
-  double Nk = Lq[qa * n1 + ka] * Lq[qb * n1 + kb] * Lq[qc * n1 + kc];
-  P[t] = Nj * Nk;
-}
-
-// Packed-symmetric DHM GEMM with the Loewdin epilogue:
-//   Keff[I, c] = sum_q P[I, q] (wq[q] V[c, q]);
-//   Hc[c][j][k] = Hc[c][k][j] = d_j (K[j][k] + Keff[I, c]) d_k, d = M^-1/2 at the cell's nodes.
-constexpr int PV_BM = 64, PV_BN = 64, PV_BK = 16;
-__global__ void __launch_bounds__(256) k_pv_gemm(
-    const double* __restrict__ P, const double* __restrict__ V, const double* __restrict__ wq,
-    const int32_t* __restrict__ pairs, const double* __restrict__ K,
-    const int32_t* __restrict__ map, const double* __restrict__ minvsqrt,
-    double* __restrict__ Hc, int64_t Msym, int64_t Nc, int nq, int nc) {
-  __shared__ double As[PV_BK][PV_BM + 1];
-  __shared__ double Bs[PV_BK][PV_BN + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int64_t I0 = blockIdx.x * (int64_t)PV_BM;
-  const int64_t c0 = blockIdx.y * (int64_t)PV_BN;
-  double acc[4][4] = {};
-  for (int q0 = 0; q0 < nq; q0 += PV_BK) {
-    for (int e = threadIdx.x; e < PV_BK * PV_BM; e += 256) {
-      int kk = e % PV_BK, i = e / PV_BK;
-      int64_t I = I0 + i;
-      int q = q0 + kk;
-      As[kk][i] = (I < Msym && q < nq) ? P[I * nq + q] : 0.0;
-      int64_t c = c0 + i;
-      Bs[kk][i] = (c < Nc && q < nq) ? V[c * nq + q] * wq[q] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < PV_BK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+// Dense cell matrices H~^c = D_c^-1/2 (K^c + V^c) D_c^-1/2 from the tensor-product form of Eq.
+// quadLocal: with B[q][aa'] = l_a(x_q) l_a'(x_q) / sqrt(w^_a w^_a') (pairs a <= a', w^ the
+// assembled 1D weights) and v = w_q w_q' w_q'' V,
+//   V^c[(abc), (a'b'c')] = sum_qx,qy,qz B[qx][aa'] B[qy][bb'] B[qz][cc'] v[qz][qy][qx],
+// one axis at a time: per pair cc' the sums over qz, qx and qy, then the two (N^2 x N^2) blocks
+// (c, c') and (c', c) are written in runs of N^2 with the kinetic term added.  About 200,000
+// multiply-adds per cell at p = 6 against 20 million for the product table times V of Eq.
+// gemmLoc (and no 162 MB table), so the writes of the matrices bound it.  One CTA takes one
+// cell and every gridDim.y-th pair cc'.
+struct CellTab {
+  const double* B;        // nq1 x npair
+  const double* K;        // N x N: the 1D kinetic matrix without its mesh factor
+  const double* om;       // N: w_a / w^_a
+  double kx, ky, kz;      // 1/2 (2/h_d)^2
+};
+__global__ void __launch_bounds__(256) k_cell_matrices(const double* __restrict__ v, CellTab tab, int N, int nq,
+                                                       int nodal, double* __restrict__ Hc) {
+  extern __shared__ double cms[];
+  const int np = N * (N + 1) / 2, n2 = N * N, nc = n2 * N;
+  double* sv = cms;                        // nq^3
+  double* sB = sv + nq * nq * nq;          // nq x np
+  double* sK = sB + nq * np;               // n2
+  double* som = sK + n2;                   // N
+  double* t1 = som + N;                    // nq x nq (qy, qx)
+  double* t2 = t1 + nq * nq;               // np x nq (aa', qy)
+  double* t3 = t2 + np * nq;               // np x np (aa', bb')
+  uint8_t* pr = reinterpret_cast<uint8_t*>(t3 + np * np);   // n2: pair index of (a, a')
+  const int64_t cell = blockIdx.x;
+  for (int t = threadIdx.x; t < nq * nq * nq; t += 256) sv[t] = v[cell * nq * nq * nq + t];
+  for (int t = threadIdx.x; t < nq * np; t += 256) sB[t] = tab.B[t];
+  for (int t = threadIdx.x; t < n2; t += 256) {
+    sK[t] = tab.K[t];
+    const int a = min(t / N, t % N), b = max(t / N, t % N);
+    pr[t] = (uint8_t)(a * N - a * (a - 1) / 2 + b - a);
   }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int64_t I = I0 + ty * 4 + i;
-    if (I >= Msym) continue;
-    int jn = pairs[2 * I], kn = pairs[2 * I + 1];
-    double kv = K[(int64_t)jn * nc + kn];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int64_t c = c0 + tx * 4 + j;
-      if (c >= Nc) continue;
-      double dj = minvsqrt[map[c * nc + jn]];
-      double dk = minvsqrt[map[c * nc + kn]];
-      double v = dj * (kv + acc[i][j]) * dk;
-      double* H = Hc + c * (int64_t)nc * nc;
-      H[(int64_t)jn * nc + kn] = v;
-      if (jn != kn) H[(int64_t)kn * nc + jn] = v;
+  for (int t = threadIdx.x; t < N; t += 256) som[t] = tab.om[t];
+  __syncthreads();
+  double* H = Hc + cell * (int64_t)nc * nc;
+  int c = 0, cp = 0;
+  for (int P = 0; P < np; ++P, ++cp) {
+    if (cp == N) {
+      ++c;
+      cp = c;
     }
+    if (P % (int)gridDim.y != (int)blockIdx.y) continue;
+    if (!nodal) {
+      for (int t = threadIdx.x; t < nq * nq; t += 256) {
+        double s = 0.0;
+        for (int q = 0; q < nq; ++q) s = fma(sB[q * np + P], sv[q * nq * nq + t], s);
+        t1[t] = s;
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < np * nq; t += 256) {
+        const int a = t / nq, qy = t - a * nq;
+        double s = 0.0;
+        for (int q = 0; q < nq; ++q) s = fma(sB[q * np + a], t1[qy * nq + q], s);
+        t2[t] = s;
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < np * np; t += 256) {
+        const int a = t / np, b = t - a * np;
+        double s = 0.0;
+        for (int q = 0; q < nq; ++q) s = fma(sB[q * np + b], t2[a * nq + q], s);
+        t3[t] = s;
+      }
+      __syncthreads();
+    }
+    // rows (a, b, c), columns (a', b', c'), and the transposed block
+    for (int t = threadIdx.x; t < n2 * n2; t += 256) {
+      const int r = t / n2, k = t - r * n2;
+      const int b = r / N, a = r - b * N, b2 = k / N, a2 = k - b2 * N;
+      double h = nodal ? 0.0 : t3[pr[a * N + a2] * np + pr[b * N + b2]];
+      if (c == cp) {
+        if (nodal && r == k) h = sv[c * n2 + r];
+        if (b == b2) h = fma(tab.kx * sK[a * N + a2], som[b] * som[c], h);
+        if (a == a2) h = fma(tab.ky * sK[b * N + b2], som[a] * som[c], h);
+      }
+      if (r == k) h = fma(tab.kz * sK[c * N + cp], som[a] * som[b], h);
+      H[(int64_t)(c * n2 + r) * nc + cp * n2 + k] = h;
+      if (c != cp) H[(int64_t)(cp * n2 + r) * nc + c * n2 + k] = h;
+    }
+    __syncthreads();
   }
 }
 
@@ -365,52 +373,8 @@ static dftfe_ham create_ham(dftfe_mesh m, void* stream, dftfe_ham src) {
       }
       h->d_colour_cells = dev_upload(flat, s);
     }
-    // a2 reference-cell tables: stiffness (Kronecker form of the GLL quadrature) and P
+    // a2 reference tables: the basis at the quadrature points (density)
     {
-      const auto& w = m->gll.w;
-      const auto& D = m->D;
-      std::vector<double> k1[3], mm1[3];
-      for (int a = 0; a < 3; ++a) {
-        k1[a].assign(n1 * n1, 0.0);
-        mm1[a].assign(n1, 0.0);
-        for (int i = 0; i < n1; ++i) {
-          mm1[a][i] = m->h[a] / 2.0 * w[i];
-          for (int j = 0; j < n1; ++j) {
-            double s1 = 0.0;
-            for (int q = 0; q < n1; ++q) s1 += w[q] * D[q * n1 + i] * D[q * n1 + j];
-            k1[a][i * n1 + j] = 2.0 / m->h[a] * s1;
-          }
-        }
-      }
-      std::vector<double> K((size_t)nc * nc, 0.0);
-      for (int j = 0; j < nc; ++j) {
-        int a = j % n1, b = (j / n1) % n1, c = j / (n1 * n1);
-        for (int k = 0; k < nc; ++k) {
-          int d = k % n1, e = (k / n1) % n1, f = k / (n1 * n1);
-          double v = 0.0;
-          if (b == e && c == f) v += k1[0][a * n1 + d] * mm1[1][b] * mm1[2][c];
-          if (a == d && c == f) v += mm1[0][a] * k1[1][b * n1 + e] * mm1[2][c];
-          if (a == d && b == e) v += mm1[0][a] * mm1[1][b] * k1[2][c * n1 + f];
-          K[(size_t)j * nc + k] = 0.5 * v;
-        }
-      }
-      h->d_K = dev_upload(K, s);
-      const int64_t Msym = (int64_t)nc * (nc + 1) / 2;
-      std::vector<int32_t> pairs(2 * Msym);
-      int64_t I = 0;
-      for (int j = 0; j < nc; ++j)
-        for (int k = j; k < nc; ++k) {
-          pairs[2 * I] = j;
-          pairs[2 * I + 1] = k;
-          ++I;
-        }
-      h->d_pairs = dev_upload(pairs, s);
-      std::vector<double> wq(m->nq);
-      for (int q = 0; q < m->nq; ++q) {
-        int qa = q % m->nq1, qb = (q / m->nq1) % m->nq1, qc = q / (m->nq1 * m->nq1);
-        wq[q] = m->quad.w[qa] * m->quad.w[qb] * m->quad.w[qc] * m->detJ;
-      }
-      h->d_wq = dev_upload(wq, s);
       std::vector<double> Nq((size_t)m->nq * nc);
       for (int q = 0; q < m->nq; ++q) {
         const int qa = q % m->nq1, qb = (q / m->nq1) % m->nq1, qc = q / (m->nq1 * m->nq1);
@@ -420,15 +384,8 @@ static dftfe_ham create_ham(dftfe_mesh m, void* stream, dftfe_ham src) {
         }
       }
       h->d_Nq = dev_upload(Nq, s);
-      if (!src) {
-        double* d_Lq = dev_upload(m->Lq, s);
-        DFTFE_CHECK_CUDA(cudaMalloc(&h->d_P, sizeof(double) * Msym * m->nq));
-        DFTFE_LAUNCH(k_products, nblk(Msym * m->nq), 256, 0, s, h->d_P, h->d_pairs, d_Lq, Msym,
-                     m->nq1, n1);
-        DFTFE_CHECK_CUDA(cudaStreamSynchronize(s));
-        cudaFree(d_Lq);
-      }
     }
+    if (!src) sf_init(h);
     if (!src) DFTFE_CHECK_CUDA(cudaMalloc(&h->d_Hc, sizeof(double) * m->Nc * (int64_t)nc * nc));
   } catch (...) {
     h->local_src = nullptr;
@@ -463,12 +420,18 @@ extern "C" dftfe_status dftfe_ham_set_potential(dftfe_ham h, const double* v_qua
   if (h->local_src)
     throw Error(DFTFE_ERR_STATE, "this ham uses another ham's local operator: set the potential on that ham");
   auto* m = h->mesh;
-  const int64_t Msym = (int64_t)m->nc * (m->nc + 1) / 2;
-  dim3 grid((unsigned)((Msym + PV_BM - 1) / PV_BM), (unsigned)((m->Nc + PV_BN - 1) / PV_BN));
+  sf_set_potential(h, v_quad);
   {
     ProfScope ps(h, "dhm_gemm");
-    DFTFE_LAUNCH(k_pv_gemm, grid, 256, 0, h->stream, h->d_P, v_quad, h->d_wq, h->d_pairs, h->d_K,
-                 h->d_map, h->d_minvsqrt, h->d_Hc, Msym, m->Nc, m->nq, m->nc);
+    const int N = m->n1, np = N * (N + 1) / 2, nq = m->nq1;
+    const CellTab tab{h->d_celltab, h->d_celltab + nq * np, h->d_celltab + nq * np + N * N,
+                      2.0 / (m->h[0] * m->h[0]), 2.0 / (m->h[1] * m->h[1]), 2.0 / (m->h[2] * m->h[2])};
+    const size_t sh = sizeof(double) * ((size_t)nq * nq * nq + nq * np + N * N + N + nq * nq + np * nq + np * np) +
+                      (size_t)N * N;
+    // enough CTAs for a few per SM when there are few cells
+    const int split = (int)std::max<int64_t>(1, std::min<int64_t>(np, 6LL * h->sm_count / m->Nc));
+    DFTFE_LAUNCH(k_cell_matrices, dim3((unsigned)m->Nc, (unsigned)split), 256, sh, h->stream, h->d_sfv, tab, N, nq,
+                 m->vquad == 1 ? 1 : 0, h->d_Hc);
   }
   h->has_potential = true;
   h->potential_version++;
@@ -557,8 +520,9 @@ extern "C" dftfe_status dftfe_ham_destroy(dftfe_ham h) {
   if (h->h_pass) cudaFreeHost(h->h_pass);
   free_nonlocal(h);
   cudaFree(h->d_map); cudaFree(h->d_mass); cudaFree(h->d_minvsqrt);
-  cudaFree(h->d_colour_cells); cudaFree(h->d_node_ptr); cudaFree(h->d_node_slot); cudaFree(h->d_K); cudaFree(h->d_P); cudaFree(h->d_pairs);
-  cudaFree(h->d_wq); cudaFree(h->d_Hc); cudaFree(h->d_Nq); cudaFree(h->d_ktab); cudaFree(h->d_ktab32);
+  cudaFree(h->d_colour_cells); cudaFree(h->d_node_ptr); cudaFree(h->d_node_slot); 
+  cudaFree(h->d_sfw); cudaFree(h->d_sfv);
+  cudaFree(h->d_celltab); cudaFree(h->d_Hc); cudaFree(h->d_Nq); cudaFree(h->d_ktab); cudaFree(h->d_ktab32);
   for (auto& kv : h->ws) kv.second.release();
   for (auto& kv : h->timers)
     for (auto& ev : kv.second.events) {

@@ -1,0 +1,114 @@
+"""The tensor-product form of the local operator against the FP64 oracle's dense cell
+matrices: every degree, both quadrature rules, anisotropic boxes with even, odd and
+two-cell axes, column counts around the kernels' tiles (several cells per CTA below 8 columns,
+ragged tiles, more than one face-buffer chunk); meshes whose quadrature rule has no such form
+keep the dense products.  Tolerance: both sides are FP64 sums of the same products in another
+order, so the parity tests' 1e-12 of the largest entry."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def dg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2203_07820_gb300 as dg
+    return dg
+
+
+def _system(dg, L, n, p, vquad=0, nq1d=0, seed=1):
+    s = synth.Stream(seed)
+    cent = np.array([[Ld * s.uniform() for Ld in L] for _ in range(3)])
+    om = oracle.PeriodicMesh(L, n, p, **({"nq1d": nq1d} if nq1d else {}))
+    oh = oracle.Hamiltonian(om, vquad=vquad)
+    mesh = dg.dftfe_mesh_create(L, n, p, vquad=vquad, nq1d=nq1d)
+    ham = dg.dftfe_ham_create(mesh)
+    v = synth.gaussian_wells(om.quad_xyz(vquad).reshape(-1, 3), cent, 2.0, 1.0, np.array(L))
+    oh.set_potential(v)
+    dg.dftfe_ham_set_potential(ham, torch.from_numpy(np.ascontiguousarray(v).reshape(-1)).cuda())
+    return om, oh, mesh, ham
+
+
+def _destroy(dg, mesh, ham):
+    dg.dftfe_ham_destroy(ham)
+    dg.dftfe_mesh_destroy(mesh)
+
+
+@pytest.mark.parametrize("vquad", [0, 1])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_apply_and_cell_matrices(dg, p, vquad):
+    n = (3, 2, 4) if p <= 5 else (2, 3, 2)
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 6.5), n, p, vquad)
+    try:
+        out = torch.empty((om.ncells, om.nodes_per_cell, om.nodes_per_cell), dtype=torch.float64, device="cuda")
+        dg.dftfe_ham_export(ham, c0=0, cell_mats=out)
+        ref = np.asarray(oh.cell_matrices())
+        assert np.abs(out.cpu().numpy() - ref).max() <= 1e-13 * np.abs(ref).max()
+        for ncol in (1, 2, 3, 7, 9, 33, 130):
+            X0 = synth.random_block(50 + ncol, om.ndofs, ncol)
+            X = torch.from_numpy(X0).cuda()
+            Y = torch.full_like(X, float("nan"))
+            dg.dftfe_ham_apply(ham, X, Y)
+            ref = oh.apply(X0)
+            err = np.abs(Y.cpu().numpy() - ref).max()
+            assert err <= TOL * np.abs(ref).max(), (ncol, err)
+    finally:
+        _destroy(dg, mesh, ham)
+
+
+@pytest.mark.parametrize("p,nq1d", [(3, 6), (4, 3), (6, 9)])
+def test_other_quadrature_rules_keep_the_dense_products(dg, p, nq1d):
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 6.5), (3, 2, 2), p, 0, nq1d)
+    try:
+        for ncol in (1, 4, 37):
+            X0 = synth.random_block(60 + ncol, om.ndofs, ncol)
+            X = torch.from_numpy(X0).cuda()
+            Y = torch.full_like(X, float("nan"))
+            dg.dftfe_ham_apply(ham, X, Y)
+            ref = oh.apply(X0)
+            assert np.abs(Y.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max(), ncol
+    finally:
+        _destroy(dg, mesh, ham)
+
+
+def test_batch_of_both_forms_is_bit_identical_to_single_passes(dg):
+    """Tensor-product systems of two degrees, a dense one (other quadrature rule) and narrow
+    blocks in one FP64 batch."""
+    specs = [((5.0, 4.0, 6.5), (3, 2, 4), 4, 0, 0, 12, 5), ((4.0, 4.0, 4.0), (2, 2, 2), 6, 1, 0, 9, 9),
+             ((5.0, 4.0, 5.0), (2, 3, 2), 3, 0, 5, 10, 4), ((4.0, 5.0, 4.0), (2, 2, 3), 4, 0, 0, 6, 2)]
+    made = [_system(dg, *s[:5], seed=i) for i, s in enumerate(specs)]
+    batch = dg.dftfe_batch_create([m[3] for m in made])
+    try:
+        X1, X2, bd1, bd2, ev, rs, deg = [], [], [], [], [], [], []
+        for i, ((om, oh, mesh, ham), s) in enumerate(zip(made, specs)):
+            N = s[5]
+            x = torch.from_numpy(synth.random_block(80 + i, om.ndofs, N)).cuda()
+            X1.append(x)
+            X2.append(x.clone())
+            b = dg.dftfe_spectrum_bounds(ham, 12, 3, N)
+            bd1.append(b)
+            bd2.append(dg.make_bounds(b.a, b.b, b.a0))
+            ev.append(torch.empty(N, dtype=torch.float64, device="cuda"))
+            rs.append(torch.empty_like(ev[-1]))
+            deg.append(5 + i)
+        blocks = [s[6] for s in specs]
+        for _ in range(2):
+            dg.dftfe_batch_chfsi_pass(batch, X1, blocks, deg, bd1, ev, rs)
+            for i, m in enumerate(made):
+                dg.dftfe_chfsi_pass(m[3], X2[i], blocks[i], deg[i], bd2[i], ev[i], rs[i])
+        for a, b in zip(X1, X2):
+            assert torch.equal(a, b)
+    finally:
+        dg.dftfe_batch_destroy(batch)
+        for m in made:
+            _destroy(dg, m[2], m[3])
