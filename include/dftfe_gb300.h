@@ -545,8 +545,8 @@ dftfe_status dftfe_profile_query(dftfe_ham ham, const char* kernel, double* tota
                                  int64_t* launches);
 
 /* Test hook for the bounded device waits (no counterpart in the paper).  The dense subspace
- * eigensolver (Rayleigh-Ritz, a cooperative launch whose CTAs meet at a grid barrier after
- * every Jacobi round) gives up a wait after a spin limit of about a second, records
+ * eigensolver (Rayleigh-Ritz, a cooperative launch whose CTAs meet at a grid barrier for
+ * every column it reduces) gives up a wait after a spin limit of about a second, records
  * DFTFE_ERR_TIMEOUT, lets every CTA return and leaves the context usable; the calling entry
  * point then returns DFTFE_ERR_TIMEOUT with X unchanged.  spin_limit > 0 replaces that limit
  * (iterations of a ~64 ns sleep; 0 restores the default) and withhold_arrival = 1 makes the

@@ -343,6 +343,11 @@ int fp64_row_splits(dftfe_ham h, int64_t ctas, int nc);
 bool gram_lower_tc(dftfe_ham h, const double* A, int64_t lda, const double* B, int64_t ldb, int64_t M, int N,
                    double* C, const double* dpart, int nchunk);
 
+// eig.cu: eigenvalues (unsorted, d) and eigenvectors (rows of VT) of the lower triangle of A, where
+// its rows fit into the shared memory of the GPU
+bool tridiag_applicable(dftfe_ham h, int N, bool cplx);
+template <typename C> void tridiag_eig(dftfe_ham h, const C* A, int N, double* d, C* VT, int* d_status);
+
 // dense.cu
 void gram_lower(dftfe_ham h, const double* A, int64_t lda, const double* B, int64_t ldb,
                 int64_t M, int N, double* C, double* part, int nsplit);

@@ -46,7 +46,8 @@ void DevBuf::release() {
 // pass they come from the batch's shared tail workspace
 static bool tail_buffer(const char* name) {
   static const char* const names[] = {"S", "Zinv", "gram_part", "Hhat", "Q", "W", "chol_d0", "chol_linv",
-                                      "eig_V", "eigz_V", "eig_vec", "eig_perm", "resid_part", "coldot_part",
+                                      "eig_V", "eigz_V", "eig_vec", "eig_perm", "eig_dc", "eig_refl", "eig_refl_z",
+                                      "eig_idx", "resid_part", "coldot_part",
                                       "gram32_part", "rotmix_Zf", "rotmix_zd", "Hz", "Qz", "rot_tc_tiles",
                                       "rot_tc_zd", "rot_tc_out", "gram_tc_part", "slices_x", "slices_xe"};
   for (const char* n : names)
