@@ -5,9 +5,8 @@
 //   1. factor the diagonal block A_kk = L_kk L_kk^T and invert it (one CTA, shared memory),
 //   2. L_ik = A_ik L_kk^-T for the blocks below it (one CTA per block),
 //   3. A_ij -= L_ik L_jk^T for the trailing lower blocks k < j <= i (one CTA per block).
-// The inverse is then formed block row by block row (block forward substitution):
-//   (L^-1)_ii = L_ii^-1,  (L^-1)_ij = -L_ii^-1 sum_{k=j}^{i-1} L_ik (L^-1)_kj   (j < i),
-// and written transposed as Z = L^-T (upper triangular), with L's strict upper triangle
+// The inverse is then formed by doubling from the inverted diagonal blocks (k_tri_inv_pair) and
+// written transposed as Z = L^-T (upper triangular), with L's strict upper triangle
 // zeroed.  A pivot not above 1e-14 times its original diagonal entry (or not finite)
 // records DFTFE_ERR_NOT_SPD; the later steps still run on finite stand-in values, so the
 // caller reads the status once after the factorisation.
@@ -37,52 +36,54 @@ __global__ void k_chol_save_diag(const double* __restrict__ A, int N, double* __
   if (i == 0) *status = 0;
 }
 
-// step 1: factor and invert the diagonal block k
+// step 1: factor and invert the diagonal block k.  Column by column, with the inverse formed alongside
+// (right-looking forward substitution on the identity): one reciprocal square root per column and no
+// division, since the FP64 pipe's latency sets the pace (80 us a block with a division per
+// entry and one thread per column of the inverse).
 __global__ void __launch_bounds__(256) k_chol_diag(double* __restrict__ A, int N, int k, const double* __restrict__ d0,
                                                    double* __restrict__ Linv, int* status) {
   using namespace chol;
   __shared__ double a[NB][NB + 1];
   __shared__ double y[NB][NB + 1];
-  __shared__ double piv;
+  __shared__ double rpiv;
   const int nb = rows_of(k, N), off = k * NB;
   load_block(A, N, k, k, a);
+  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) y[t / NB][t % NB] = t / NB == t % NB ? 1.0 : 0.0;
   __syncthreads();
   for (int j = 0; j < nb; ++j) {
     if (threadIdx.x == 0) {
       const double d = a[j][j], dorig = d0[off + j];
       if (!(d > 1e-14 * dorig) || !(dorig > 0.0) || !isfinite(d)) {
         atomicExch(status, (int)DFTFE_ERR_NOT_SPD);
-        piv = 1.0;                                    // finite stand-in; the status stays set
+        rpiv = 1.0;                                   // finite stand-in; the status stays set
+        a[j][j] = 1.0;
       } else {
-        piv = sqrt(d);
+        rpiv = rsqrt(d);
+        a[j][j] = d * rpiv;
       }
-      a[j][j] = piv;
     }
     __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) a[i][j] /= piv;
+    if (threadIdx.x < NB) {
+      const int i = threadIdx.x;
+      if (i > j && i < nb) a[i][j] *= rpiv;
+    } else if (threadIdx.x < 2 * NB) {
+      const int c = threadIdx.x - NB;
+      if (c <= j) y[j][c] *= rpiv;
+    }
     __syncthreads();
-    // trailing update of the block's lower triangle
+    // trailing lower triangle of the block, and the rows of the inverse below j
     const int m = nb - j - 1;
-    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-      const int i = j + 1 + t / m, l = j + 1 + t % m;
-      if (l <= i) a[i][l] -= a[i][j] * a[l][j];
+    for (int t = threadIdx.x; t < m * NB; t += blockDim.x) {
+      const int i = j + 1 + t / NB, l = t % NB;
+      const double lij = a[i][j];
+      if (l > j) {
+        if (l <= i) a[i][l] = fma(-lij, a[l][j], a[i][l]);
+      } else {
+        y[i][l] = fma(-lij, y[j][l], y[i][l]);
+      }
     }
     __syncthreads();
   }
-  // L_kk^-1 column by column (thread c solves L y = e_c by forward substitution)
-  if (threadIdx.x < NB) {
-    const int c = threadIdx.x;
-    for (int i = 0; i < NB; ++i) {
-      double v = 0.0;
-      if (c < nb && i < nb && i >= c) {
-        double s = (i == c) ? 1.0 : 0.0;
-        for (int l = c; l < i; ++l) s -= a[i][l] * y[l][c];
-        v = s / a[i][i];
-      }
-      y[i][c] = v;
-    }
-  }
-  __syncthreads();
   for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
     const int r = t / NB, c = t % NB;
     if (r < nb && c < nb) {
@@ -137,38 +138,37 @@ __global__ void __launch_bounds__(256) k_chol_update(double* __restrict__ A, int
   }
 }
 
-// inverse, block row i: (L^-1)_ij = -L_ii^-1 sum_{k=j}^{i-1} L_ik (L^-1)_kj, j = blockIdx.x < i
-__global__ void __launch_bounds__(256) k_tri_inv_row(const double* __restrict__ L, int N, int i,
-                                                     double* __restrict__ Linv) {
-  using namespace chol;
-  __shared__ double lk[NB][NB + 1];
-  __shared__ double vk[NB][NB + 1];
-  __shared__ double acc[NB][NB + 1];
-  const int j = blockIdx.x;
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) acc[e / NB][e % NB] = 0.0;
-  for (int k = j; k < i; ++k) {
+// inverse by doubling: with the diagonal blocks of h rows inverted, pairs of them give
+//   [[A, 0], [C, B]]^-1 = [[A^-1, 0], [-B^-1 C A^-1, B^-1]],
+// two products per doubling (PHASE 0: T = C A^-1, PHASE 1: -B^-1 T), each spread over 16 x 16 tiles
+// on all SMs (a block row at a time, one CTA per block of the row, took N / 32 launches of up to N / 32
+// serial 32^3 products: 1.14 ms at N = 512).
+constexpr int TI = 16;
+template <int PHASE>
+__global__ void __launch_bounds__(TI * TI) k_tri_inv_pair(const double* __restrict__ L, int N, int h,
+                                                          double* __restrict__ Linv, double* __restrict__ T) {
+  __shared__ double p[TI][TI + 1];
+  __shared__ double q[TI][TI + 1];
+  const int s = 2 * h * blockIdx.x, mid = s + h, r0 = mid + TI * blockIdx.y, c0 = s + TI * blockIdx.z;
+  if (mid >= N || r0 >= min(N, mid + h)) return;
+  const int tr = threadIdx.x / TI, tc = threadIdx.x % TI;
+  const int r = r0 + tr, c = c0 + tc, end = min(N, mid + h);
+  // PHASE 0: sum over k in [s, mid), A^-1 lower: k >= c0; PHASE 1: k in [mid, end), B^-1 lower: k <= r0 + 15
+  const int k0 = PHASE == 0 ? c0 : mid, k1 = PHASE == 0 ? mid : min(end, r0 + TI);
+  double acc = 0.0;
+  for (int k = k0; k < k1; k += TI) {
+    const double* P = PHASE == 0 ? L : Linv;
+    const double* Q = PHASE == 0 ? Linv : T;
+    p[tr][tc] = r < end && k + tc < k1 ? P[(int64_t)r * N + k + tc] : 0.0;
+    q[tr][tc] = k + tr < k1 ? Q[(int64_t)(k + tr) * N + c] : 0.0;
     __syncthreads();
-    load_block(L, N, i, k, lk);
-    load_block(Linv, N, k, j, vk);
+#pragma unroll
+    for (int l = 0; l < TI; ++l) acc = fma(p[tr][l], q[l][tc], acc);
     __syncthreads();
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-      const int r = e / NB, c = e % NB;
-      double s = acc[r][c];
-#pragma unroll 8
-      for (int l = 0; l < NB; ++l) s = fma(lk[r][l], vk[l][c], s);
-      acc[r][c] = s;
-    }
   }
-  __syncthreads();
-  load_block(Linv, N, i, i, lk);
-  __syncthreads();
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, c = e % NB;
-    double s = 0.0;
-#pragma unroll 8
-    for (int l = 0; l <= r; ++l) s = fma(lk[r][l], acc[l][c], s);
-    const int gi = i * NB + r, gj = j * NB + c;
-    if (gi < N && gj < N) Linv[(int64_t)gi * N + gj] = -s;
+  if (r < end) {
+    if (PHASE == 0) T[(int64_t)r * N + c] = acc;
+    else Linv[(int64_t)r * N + c] = -acc;
   }
 }
 
@@ -206,7 +206,12 @@ void tri_inverse_blocked(dftfe_ham h, double* L, double* Z, int N) {
   const int nbk = (N + NB - 1) / NB;
   double* Linv = (double*)ws_get(h, "chol_linv", sizeof(double) * (size_t)N * N);
   ProfScope ps(h, "trtri");
-  for (int i = 1; i < nbk; ++i) DFTFE_LAUNCH(k_tri_inv_row, i, 256, 0, s, L, N, i, Linv);
+  for (int hb = 1; hb < nbk; hb *= 2) {           // Z is the scratch of the products until it is written
+    const int hh = hb * NB;
+    const dim3 grid((unsigned)((N + 2 * hh - 1) / (2 * hh)), (unsigned)(hh / TI), (unsigned)(hh / TI));
+    DFTFE_LAUNCH(k_tri_inv_pair<0>, grid, TI * TI, 0, s, L, N, hh, Linv, Z);
+    DFTFE_LAUNCH(k_tri_inv_pair<1>, grid, TI * TI, 0, s, L, N, hh, Linv, Z);
+  }
   DFTFE_LAUNCH(k_tri_finish, nblk_c((int64_t)N * N), 256, 0, s, L, Linv, Z, N);
 }
 

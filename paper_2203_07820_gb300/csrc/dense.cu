@@ -10,8 +10,8 @@
 //  syevd        H^ = Q Theta Q^T: eig.cu (beyond its shared-memory rows, about 1,700 columns, a
 //               parallel cyclic Jacobi in one cooperative launch), then ascending sort and the
 //               sign convention (step 2b-c); syevd_z is the Hermitian form for Bloch k-points.
-//  tridiag_ql   implicit-shift QL on a tridiagonal (Bowdler, Martin, Reinsch, Wilkinson,
-//               Numer. Math. 11, 1968), for the Lanczos bound.
+//  lanczos      k steps with full reorthogonalisation; the ends of the tridiagonal spectrum by
+//               Sturm counts (a7).
 //  residuals    ||W_i - theta_i X_i|| or the generalised form (a13), real or complex.
 #include "internal.h"
 #include "gridbar.h"
@@ -42,7 +42,9 @@ __device__ double block_sum(double v, double* red) {
 }
 
 // ------------------------------------------------------------------ Gram
-constexpr int GT = 64, GK = 16;
+// GT x GT tiles: 64, or 32 where 64 would leave much of a tile outside the block of columns.
+constexpr int GK = 16;
+template <int GT>
 __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__ A, int64_t lda,
                                                       const double* __restrict__ B, int64_t ldb,
                                                       int64_t M, int N, int64_t rows_per_split,
@@ -59,7 +61,8 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
   const int64_t m0 = (int64_t)blockIdx.y * rows_per_split;
   const int64_t m1 = min(M, m0 + rows_per_split);
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4] = {};
+  constexpr int TE = GT / 16;
+  double acc[TE][TE] = {};
   for (int64_t mm = m0; mm < m1; mm += GK) {
     for (int e = threadIdx.x; e < GK * GT; e += 256) {
       const int kk = e / GT, c = e % GT;
@@ -71,48 +74,62 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < GK; ++kk) {
-      double a[4], b[4];
+      double a[TE], b[TE];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < TE; ++i) a[i] = As[kk][ty + 16 * i];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+      for (int j = 0; j < TE; ++j) b[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TE; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < TE; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
     }
     __syncthreads();
   }
   double* out = part + (int64_t)blockIdx.y * N * N;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < TE; ++i) {
     const int gi = i0 + ty + 16 * i;
     if (gi >= N) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < TE; ++j) {
       const int gj = j0 + tx + 16 * j;
       if (gj < N) out[(int64_t)gi * N + gj] = acc[i][j];
     }
   }
 }
 
-// C[i][j] = C[j][i] = sum_s part[s][i][j] for i >= j (fixed order over s).
-__global__ void k_gram_reduce(const double* __restrict__ part, int nsplit, int N, double* __restrict__ C) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)N * N) return;
+// C[i][j] = C[j][i] = sum_s part[s][i][j] for i >= j, eight lanes per entry (each every eighth split, then
+// a fixed tree), so that many splits are not one chain of loads.
+__global__ void __launch_bounds__(256) k_gram_reduce(const double* __restrict__ part, int nsplit, int N,
+                                                     double* __restrict__ C) {
+  const int64_t t = blockIdx.x * (int64_t)32 + (threadIdx.x & 31);
+  const int lane8 = threadIdx.x >> 5;
+  __shared__ double red[8][32];
   const int i = (int)(t / N), j = (int)(t % N);
-  if (i < j) return;
+  const bool ok = t < (int64_t)N * N && i >= j;
   double s = 0.0;
-  for (int k = 0; k < nsplit; ++k) s += part[(int64_t)k * N * N + t];
+  if (ok)
+    for (int k = lane8; k < nsplit; k += 8) s += part[(int64_t)k * N * N + t];
+  red[lane8][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (lane8 || !ok) return;
+  const int l = threadIdx.x;
+  s = ((red[0][l] + red[1][l]) + (red[2][l] + red[3][l])) + ((red[4][l] + red[5][l]) + (red[6][l] + red[7][l]));
   C[(int64_t)i * N + j] = s;
   C[(int64_t)j * N + i] = s;
 }
 
+// 64-column tiles unless 32-column ones cover at least a fifth less of the matrix
+static int gram_tile(int N) {
+  const int64_t t64 = (N + 63) / 64, t32 = (N + 31) / 32;
+  return 32 * 32 * t32 * (t32 + 1) < 0.8 * 64 * 64 * t64 * (t64 + 1) ? 32 : 64;
+}
 int gram_nsplit(dftfe_ham h, int64_t M, int N) {
-  const int T = (N + GT - 1) / GT;
+  const int GT = gram_tile(N), T = (N + GT - 1) / GT;
   const int ntiles = T * (T + 1) / 2;
   int64_t want = (4LL * h->sm_count + ntiles - 1) / ntiles;
-  int64_t maxs = std::max<int64_t>(1, M / 256);
+  int64_t maxs = std::max<int64_t>(1, M / 64);
   return (int)std::max<int64_t>(1, std::min(want, maxs));
 }
 
@@ -120,15 +137,17 @@ void gram_lower(dftfe_ham h, const double* A, int64_t lda, const double* B, int6
                 int N, double* C, double* part, int nsplit) {
   // no host data: the kernel decodes its tile from the block index, so the launch can be
   // captured in a CUDA graph and replayed
-  const int T = (N + GT - 1) / GT;
+  const int GT = gram_tile(N), T = (N + GT - 1) / GT;
   const int ntiles = T * (T + 1) / 2;
-  const int64_t rows = (M + nsplit - 1) / nsplit;
+  const int64_t rows = ((M + nsplit - 1) / nsplit + GK - 1) / GK * GK;   // whole chunks; a split may be empty
   {
     ProfScope ps(h, "gram");
-    DFTFE_LAUNCH(k_gram_partial, dim3(ntiles, nsplit), 256, 0, h->stream, A, lda, B, ldb, M, N,
-                 rows, part);
+    if (GT == 32)
+      DFTFE_LAUNCH(k_gram_partial<32>, dim3(ntiles, nsplit), 256, 0, h->stream, A, lda, B, ldb, M, N, rows, part);
+    else
+      DFTFE_LAUNCH(k_gram_partial<64>, dim3(ntiles, nsplit), 256, 0, h->stream, A, lda, B, ldb, M, N, rows, part);
   }
-  DFTFE_LAUNCH(k_gram_reduce, nblk((int64_t)N * N), 256, 0, h->stream, part, nsplit, N, C);
+  DFTFE_LAUNCH(k_gram_reduce, nblk((int64_t)N * N, 32), 256, 0, h->stream, part, nsplit, N, C);
 }
 
 // ---------------------------------------------------------------- Cholesky
@@ -458,127 +477,6 @@ __global__ void k_fro_norm(const double* __restrict__ A, int N, double* out) {
   if (threadIdx.x == 0) *out = sqrt(s);
 }
 
-// Implicit QL with Wilkinson shifts on (d, e); rotations are replayed on the rows of Z
-// this CTA holds in shared memory.  Every CTA runs the same scalar recurrence (lane 0),
-// so all agree on d; CTA 0 writes it back.
-__global__ void __launch_bounds__(32) k_tql(double* __restrict__ dg, double* __restrict__ eg,
-                                            double* __restrict__ Z, int N, int R, int* status) {
-  extern __shared__ double sm[];
-  double* d = sm;                 // N
-  double* e = d + N;              // N
-  double* cs = e + N;             // N
-  double* sn = cs + N;            // N
-  double* zr = sn + N;            // R x (N+1)
-  __shared__ int nrot, base, fail;
-  const int r0 = blockIdx.x * R;
-  const int myrow = r0 + threadIdx.x;
-  const bool have = threadIdx.x < R && myrow < N;
-  for (int i = threadIdx.x; i < N; i += 32) {
-    d[i] = dg[i];
-    e[i] = (i < N - 1) ? eg[i] : 0.0;
-  }
-  for (int r = 0; r < R; ++r)
-    if (r0 + r < N)
-      for (int j = threadIdx.x; j < N; j += 32) zr[r * (N + 1) + j] = Z[(int64_t)(r0 + r) * N + j];
-  if (threadIdx.x == 0) fail = 0;
-  __syncwarp();
-  const double eps = 2.220446049250313e-16;
-  for (int l = 0; l < N; ++l) {
-    int iter = 0;
-    while (true) {
-      // lane 0 performs one QL sweep (or detects convergence) and records the rotations
-      if (threadIdx.x == 0) {
-        nrot = 0;
-        int m = l;
-        for (; m < N - 1; ++m) {
-          const double dd = fabs(d[m]) + fabs(d[m + 1]);
-          if (fabs(e[m]) <= eps * dd) break;
-        }
-        if (m == l) {
-          nrot = -1;
-        } else if (iter >= 60) {
-          nrot = -1;
-          fail = 1;
-        } else {
-          ++iter;
-          double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-          double r = sqrt(fma(g, g, 1.0));
-          g = d[m] - d[l] + e[l] / (g + copysign(r, g));
-          double s = 1.0, c = 1.0, p = 0.0;
-          int i = m - 1;
-          bool early = false;
-          for (; i >= l; --i) {
-            const double f = s * e[i], b = c * e[i];
-            // Givens rotation from (f, g): one reciprocal square root instead of a
-            // hypot and two divisions (the FP64 pipe is slow; this loop is serial)
-            const double r2 = fma(f, f, g * g);
-            if (r2 == 0.0) {
-              e[i + 1] = 0.0;
-              d[i + 1] -= p;
-              e[m] = 0.0;
-              early = true;
-              break;
-            }
-            const double rinv = rsqrt(r2);
-            r = r2 * rinv;
-            e[i + 1] = r;
-            s = f * rinv;
-            c = g * rinv;
-            g = d[i + 1] - p;
-            r = (d[i] - g) * s + 2.0 * c * b;
-            p = s * r;
-            d[i + 1] = g + p;
-            g = c * r - b;
-            cs[nrot] = c;
-            sn[nrot] = s;
-            ++nrot;
-          }
-          base = m - 1;  // rotation t acts on columns (base - t, base - t + 1)
-          if (!early) {
-            d[l] -= p;
-            e[l] = g;
-            e[m] = 0.0;
-          }
-        }
-      }
-      __syncwarp();
-      const int nr = nrot;
-      if (nr < 0) break;
-      if (have) {
-        double* z = zr + threadIdx.x * (N + 1);
-        const int b0 = base;
-        for (int t = 0; t < nr; ++t) {
-          const int i = b0 - t;
-          const double f = z[i + 1];
-          z[i + 1] = sn[t] * z[i] + cs[t] * f;
-          z[i] = cs[t] * z[i] - sn[t] * f;
-        }
-      }
-      __syncwarp();
-    }
-    if (fail) break;
-  }
-  __syncwarp();
-  if (have)
-    for (int j = 0; j < N; ++j) Z[(int64_t)myrow * N + j] = zr[threadIdx.x * (N + 1) + j];
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < N; i += 32) dg[i] = d[i];
-    if (threadIdx.x == 0) *status = fail ? (int)DFTFE_ERR_NOCONV : 0;
-  }
-}
-
-void tridiag_ql(cudaStream_t s, double* d, double* e, double* Z, int N, int* d_status) {
-  int R = (int)std::min<int64_t>(32, std::max<int64_t>(1, 131072 / ((int64_t)(N + 1) * 8)));
-  size_t sh = (size_t)(4 * N + R * (N + 1)) * sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_tql, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    attr = true;
-  }
-  if (sh > 220 * 1024) throw Error(DFTFE_ERR_ARG, "dense eigensolver: N too large");
-  DFTFE_LAUNCH(k_tql, (unsigned)((N + R - 1) / R), 32, sh, s, d, e, Z, N, R, d_status);
-}
-
 // ascending order (ties by index) and the sign convention: the largest-|.| entry of each
 // eigenvector (first one on ties) is made positive.
 // ascending order by a strict total order (NaN after every number, ties by index), so perm
@@ -794,30 +692,42 @@ void random_uniform(cudaStream_t s, double* out, int64_t n, uint64_t seed, int64
 }
 
 // ------------------------------------------------------------------ Lanczos
-constexpr int LZ_G = 512;
-// part[v*G + b] = partial dot of V[v] (stride M) with w over block b's rows.
-__global__ void __launch_bounds__(256) k_multidot_partial(const double* __restrict__ Vm, int nv,
-                                                          const double* __restrict__ w, int64_t M,
-                                                          double* __restrict__ part) {
-  __shared__ double red[9];
+constexpr int LZ_G = 304;          // CTAs of the dot products
+constexpr int LZ_W = 8;            // warps of each
+__host__ __device__ constexpr int lz_segments(int nv) { return nv >= 5 ? 1 : nv >= 3 ? 2 : nv == 2 ? 4 : 8; }
+// part[(v*G + b)*segs + q] = partial dot of V[v] (stride M) with w over segment q of block b's rows: one
+// warp per (vector, segment), so that neither one vector nor twenty leave warps idle.
+__global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* __restrict__ Vm, int nv,
+                                                                const double* __restrict__ w, int64_t M,
+                                                                double* __restrict__ part) {
+  const int segs = lz_segments(nv), lane = threadIdx.x & 31;
   const int64_t rows = (M + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = blockIdx.x * rows, i1 = min(M, i0 + rows);
-  for (int v = 0; v < nv; ++v) {
+  const int64_t i0 = blockIdx.x * rows, i1 = min(M, i0 + rows), len = (rows + segs - 1) / segs;
+  for (int t = threadIdx.x >> 5; t < nv * segs; t += LZ_W) {
+    const int v = t / segs, q = t - v * segs;
     const double* x = Vm + (int64_t)v * M;
+    const int64_t e = min(i1, i0 + (q + 1) * len);
     double s = 0.0;
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += 256) s = fma(x[i], w[i], s);
-    s = block_sum<256>(s, red);
-    if (threadIdx.x == 0) part[v * gridDim.x + blockIdx.x] = s;
+#pragma unroll 4
+    for (int64_t i = i0 + q * len + lane; i < e; i += 32) s = fma(x[i], w[i], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) part[((int64_t)v * gridDim.x + blockIdx.x) * segs + q] = s;
   }
 }
 
-// out[v] = sum_b part[v*G + b] (fixed order); mode 1 stores sqrt.
-__global__ void k_multidot_final(const double* part, int nv, int G, double* out, int mode) {
-  const int v = threadIdx.x;
-  if (v >= nv) return;
+// out[v] = sum of part's n entries of vector v = blockIdx.x (fixed order); mode 1 stores sqrt.
+__global__ void __launch_bounds__(128) k_multidot_final(const double* __restrict__ part, int n, double* out, int mode) {
+  __shared__ double red[5];
   double s = 0.0;
-  for (int b = 0; b < G; ++b) s += part[v * G + b];
-  out[v] = mode == 1 ? sqrt(s) : s;
+  for (int b = threadIdx.x; b < n; b += 128) s += part[(int64_t)blockIdx.x * n + b];
+  s = block_sum<128>(s, red);
+  if (threadIdx.x == 0) out[blockIdx.x] = mode == 1 ? sqrt(s) : s;
+}
+static void multidot(cudaStream_t s, const double* Vm, int nv, const double* w, int64_t M, double* part, double* out,
+                     int mode) {
+  DFTFE_LAUNCH(k_multidot_partial, LZ_G, 32 * LZ_W, 0, s, Vm, nv, w, M, part);
+  DFTFE_LAUNCH(k_multidot_final, (unsigned)nv, 128, 0, s, part, LZ_G * lz_segments(nv), out, mode);
 }
 
 // w = (w - a v) - b u   (a = *pa, b = *pb or 0)
@@ -847,29 +757,65 @@ __global__ void k_lz_scale(double* out, const double* w, const double* pn, int64
   out[i] = n > 0.0 ? w[i] / n : 0.0;
 }
 
-__global__ void k_lz_tridiag(const double* alpha, const double* beta, int k, double* d, double* e, double* Z) {
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+// Smallest and largest eigenvalue of the k x k tridiagonal matrix (alpha, beta) by Sturm counts: warp 0
+// the smallest, warp 1 the largest, each lane counting the eigenvalues below its own point of the
+// bracket (33 sections a step).  out3 = {theta_min, theta_max, b}, b the upper-bound estimator of
+// Zhou and Saad: the largest Ritz value plus the norm of the last Lanczos residual |beta_k|.
+// (theta_max + |beta_k| |s_k|, the residual of that Ritz pair alone, undershoots when the top of the
+// spectrum is clustered: measured on a periodic 27-cell p = 4 box, 30.21 against lambda_max = 30.54.)
+// NOCONV when the matrix is not finite.
+__global__ void __launch_bounds__(64) k_lz_bound(const double* __restrict__ alpha, const double* __restrict__ beta,
+                                                 int k, double* out3, int* status) {
+  __shared__ double d[200], e2[200];
+  __shared__ double theta[2];
+  __shared__ int bad;
+  const int lane = threadIdx.x & 31, top = threadIdx.x >> 5;
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  double lo = 1e300, hi = -1e300;
+  for (int i = threadIdx.x; i < k; i += 64) {
+    const double b = i < k - 1 ? beta[i] : 0.0;
     d[i] = alpha[i];
-    e[i] = i < k - 1 ? beta[i] : 0.0;
+    e2[i] = b * b;
+    if (!isfinite(alpha[i]) || !isfinite(beta[i]) || !isfinite(b * b)) bad = 1;
   }
-  for (int t = threadIdx.x; t < k * k; t += blockDim.x) Z[t] = (t / k == t % k) ? 1.0 : 0.0;
-}
-
-__global__ void k_lz_bound(const double* d, const double* Z, const double* beta, int k, double* out3) {
-  if (threadIdx.x != 0) return;
-  int imin = 0, imax = 0;
-  for (int i = 1; i < k; ++i) {
-    if (d[i] < d[imin]) imin = i;
-    if (d[i] > d[imax]) imax = i;
+  __syncthreads();
+  for (int i = lane; i < k; i += 32) {      // Gershgorin
+    const double r = (i > 0 ? sqrt(e2[i - 1]) : 0.0) + (i < k - 1 ? sqrt(e2[i]) : 0.0);
+    lo = fmin(lo, d[i] - r);
+    hi = fmax(hi, d[i] + r);
   }
-  out3[0] = d[imin];
-  out3[1] = d[imax];
-  // upper-bound estimator of Zhou and Saad: the largest Ritz value plus the norm of the last
-  // Lanczos residual |beta_k|.  (theta_max + |beta_k| |s_k|, the residual of that Ritz pair
-  // alone, undershoots when the top of the spectrum is clustered: measured on a periodic
-  // 27-cell p = 4 box, 30.21 against lambda_max = 30.54.)
-  (void)Z;
-  out3[2] = d[imax] + fabs(beta[k - 1]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  const double mag = fmax(fabs(lo), fabs(hi)), tiny = 1e-300 + mag * 1e-40;
+  lo -= 1e-15 * mag + tiny;
+  hi += 1e-15 * mag + tiny;
+  const int want = top ? k : 1;
+  for (int it = 0; it < 14 && !bad; ++it) {
+    const double x = lo + (hi - lo) * ((lane + 1) * (1.0 / 33.0));
+    int below = 0;
+    double q = 1.0;
+    for (int i = 0; i < k; ++i) {
+      q = d[i] - x - (i > 0 ? e2[i - 1] / q : 0.0);
+      if (fabs(q) < tiny) q = -tiny;
+      below += q < 0.0;
+    }
+    const unsigned reach = __ballot_sync(0xffffffffu, below >= want);     // the root is below these points
+    const int f = reach ? __ffs(reach) - 1 : 32;
+    const double xf = __shfl_sync(0xffffffffu, x, f < 32 ? f : 31), xp = __shfl_sync(0xffffffffu, x, f > 0 ? f - 1 : 0);
+    if (f < 32) hi = xf;
+    if (f > 0) lo = xp;
+  }
+  if (lane == 0) theta[top] = 0.5 * (lo + hi);
+  __syncthreads();
+  if (threadIdx.x) return;
+  out3[0] = theta[0];
+  out3[1] = theta[1];
+  out3[2] = theta[1] + fabs(beta[k - 1]);
+  *status = bad ? (int)DFTFE_ERR_NOCONV : 0;
 }
 
 void lanczos(dftfe_ham h, int k, const double* v0, uint64_t seed, double* out3, bool cplx) {
@@ -880,42 +826,33 @@ void lanczos(dftfe_ham h, int k, const double* v0, uint64_t seed, double* out3, 
   cudaStream_t s = h->stream;
   double* Vm = (double*)ws_get(h, "lz_V", sizeof(double) * (size_t)(k + 1) * M);
   double* w = (double*)ws_get(h, "lz_w", sizeof(double) * (size_t)M);
-  double* sc = (double*)ws_get(h, "lz_scal", sizeof(double) * (size_t)(4 * k + 8 + k * k + 2 * k));
-  double* part = (double*)ws_get(h, "lz_part", sizeof(double) * (size_t)(k + 1) * LZ_G);
+  double* sc = (double*)ws_get(h, "lz_scal", sizeof(double) * (size_t)(3 * k + 8));
+  double* part = (double*)ws_get(h, "lz_part", sizeof(double) * (size_t)(k + 8) * LZ_G);   // 8 G entries at least
   int* st = (int*)ws_get(h, "lz_status", sizeof(int));
   double* alpha = sc;
   double* beta = sc + k;
   double* hco = sc + 2 * k;        // k + 1
   double* nrm = sc + 3 * k + 1;    // 1
-  double* d = sc + 3 * k + 2;      // k
-  double* e = d + k;               // k
-  double* Z = e + k;               // k*k
-  double* d_out = Z + k * k;       // 3
+  double* d_out = sc + 3 * k + 2;  // 3
   if (v0) DFTFE_CHECK_CUDA(cudaMemcpyAsync(w, v0, sizeof(double) * M, cudaMemcpyDeviceToDevice, s));
   else random_uniform(s, w, M, seed, 0);
-  DFTFE_LAUNCH(k_multidot_partial, LZ_G, 256, 0, s, w, 1, w, M, part);
-  DFTFE_LAUNCH(k_multidot_final, 1, 32, 0, s, part, 1, LZ_G, nrm, 1);
+  multidot(s, w, 1, w, M, part, nrm, 1);
   DFTFE_LAUNCH(k_lz_scale, nblk(M), 256, 0, s, Vm, w, nrm, M);
   for (int j = 0; j < k; ++j) {
     double* vj = Vm + (int64_t)j * M;
     if (cplx) apply_combo_z(h, vj, 1, nullptr, 0, w, 1, 1, 1.0, 0.0, 0.0);
     else apply_combo(h, vj, 1, nullptr, 0, w, 1, 1, 1.0, 0.0, 0.0);
-    DFTFE_LAUNCH(k_multidot_partial, LZ_G, 256, 0, s, vj, 1, w, M, part);
-    DFTFE_LAUNCH(k_multidot_final, 1, 32, 0, s, part, 1, LZ_G, alpha + j, 0);
+    multidot(s, vj, 1, w, M, part, alpha + j, 0);
     DFTFE_LAUNCH(k_lz_three_term, nblk(M), 256, 0, s, w, vj, j > 0 ? vj - M : nullptr, alpha + j,
                  j > 0 ? beta + j - 1 : alpha + j, M);
     for (int rep = 0; rep < 2; ++rep) {
-      DFTFE_LAUNCH(k_multidot_partial, LZ_G, 256, 0, s, Vm, j + 1, w, M, part);
-      DFTFE_LAUNCH(k_multidot_final, 1, 256, 0, s, part, j + 1, LZ_G, hco, 0);
+      multidot(s, Vm, j + 1, w, M, part, hco, 0);
       DFTFE_LAUNCH(k_lz_reorth, nblk(M), 256, 0, s, w, Vm, j + 1, hco, M);
     }
-    DFTFE_LAUNCH(k_multidot_partial, LZ_G, 256, 0, s, w, 1, w, M, part);
-    DFTFE_LAUNCH(k_multidot_final, 1, 32, 0, s, part, 1, LZ_G, beta + j, 1);
+    multidot(s, w, 1, w, M, part, beta + j, 1);
     DFTFE_LAUNCH(k_lz_scale, nblk(M), 256, 0, s, Vm + (int64_t)(j + 1) * M, w, beta + j, M);
   }
-  DFTFE_LAUNCH(k_lz_tridiag, 1, 256, 0, s, alpha, beta, k, d, e, Z);
-  tridiag_ql(s, d, e, Z, k, st);
-  DFTFE_LAUNCH(k_lz_bound, 1, 32, 0, s, d, Z, beta, k, d_out);
+  DFTFE_LAUNCH(k_lz_bound, 1, 64, 0, s, alpha, beta, k, d_out, st);
   int hst = 0;
   DFTFE_CHECK_CUDA(cudaMemcpyAsync(out3, d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
   DFTFE_CHECK_CUDA(cudaMemcpyAsync(&hst, st, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -933,11 +870,11 @@ namespace dftfe {
 void gram_partial_launch(cudaStream_t s, const double* A, int64_t lda, const double* B, int64_t ldb,
                          int64_t M, int N, int nsplit, int ntiles, double* part) {
   const int64_t rows = (M + nsplit - 1) / nsplit;
-  DFTFE_LAUNCH(k_gram_partial, dim3(ntiles, nsplit), 256, 0, s, A, lda, B, ldb, M, N, rows, part);
+  DFTFE_LAUNCH(k_gram_partial<64>, dim3(ntiles, nsplit), 256, 0, s, A, lda, B, ldb, M, N, rows, part);
 }
 
 void gram_reduce_launch(cudaStream_t s, const double* part, int nsplit, int N, double* C) {
-  DFTFE_LAUNCH(k_gram_reduce, nblk((int64_t)N * N), 256, 0, s, part, nsplit, N, C);
+  DFTFE_LAUNCH(k_gram_reduce, nblk((int64_t)N * N, 32), 256, 0, s, part, nsplit, N, C);
 }
 
 template <int R, int CPT>
