@@ -1169,7 +1169,11 @@ static void apply_combo_mixed(dftfe_ham h, bool tf32, const uint8_t* A, int nkc,
       const int nb = std::min(kSfCols, ncol - c0);
       const sf::Item<float> one = sf_item32(h, v, face, X + c0, ldx, Xp ? Xp + c0 : nullptr, ldp, Z + c0, ldz, nb, alpha,
                                             s1, s2);
-      auto run = [&]() { sf_launch32(h->stream, h->sm_count, m, kpoint, one, nullptr, nullptr, sf_cell_work32(m, nb), nullptr, m->Nc); };
+      const int width = sf_width32(h->sm_count, m->n1, sf_cell_work32(m, nb, 4));
+      const int64_t nwork = sf_cell_work32(m, nb, width);
+      auto run = [&]() {
+        sf_launch32(h->stream, h->sm_count, m, kpoint, width, one, nullptr, nullptr, nwork, nullptr, m->Nc);
+      };
       if (h->autotune && !h->tuned_mixed_done && !capturing(h->stream)) {
         h->tuned_mixed = time_sf32(h->stream, run);
         h->tuned_mixed_done = true;
@@ -1300,6 +1304,7 @@ struct MixedRoundPlan {
     int k;
     const dftfe_mesh_s* mesh;
     bool kpoint;
+    int width;
     size_t item_off, cell_off, face_off;
     int nitems;
     int64_t ncell, nface;
@@ -1470,10 +1475,13 @@ static void plan_sf_round(MixedRoundPlan& R, std::vector<int2>& work, std::vecto
       const std::vector<int>& act = g.second;
       auto it = lists.find(act);
       if (it == lists.end()) {
-        MixedRoundPlan::SfLaunch L{0, R.blk[act[0]].h->mesh, R.blk[act[0]].kpoint, 0, work.size() - R.work_base, 0,
-                                   (int)act.size(), 0, 0};
+        int64_t items4 = 0;
+        for (int s : act) items4 += sf_cell_work32(R.blk[s].h->mesh, R.blk[s].ncol, 4);
+        const int width = sf_width32(R.blk[0].h->sm_count, R.blk[act[0]].h->mesh->n1, items4);
+        MixedRoundPlan::SfLaunch L{0, R.blk[act[0]].h->mesh, R.blk[act[0]].kpoint, width, 0,
+                                   work.size() - R.work_base, 0, (int)act.size(), 0, 0};
         for (size_t q = 0; q < act.size(); ++q) {
-          const int64_t n = sf_cell_work32(R.blk[act[q]].h->mesh, R.blk[act[q]].ncol);
+          const int64_t n = sf_cell_work32(R.blk[act[q]].h->mesh, R.blk[act[q]].ncol, width);
           for (int64_t t = 0; t < n; ++t) work.push_back(make_int2((int)q, (int)t));
         }
         L.face_off = work.size() - R.work_base;
@@ -1540,7 +1548,7 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
     for (; lsf < R.sf_launches.size() && R.sf_launches[lsf].k == k; ++lsf) {
       const auto& L = R.sf_launches[lsf];
       ProfScope ps(blk[0].h, "batch_cell_tf32x3");
-      sf_launch32(stream, sm, L.mesh, L.kpoint, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
+      sf_launch32(stream, sm, L.mesh, L.kpoint, L.width, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
                   d_work + R.work_base + L.cell_off, L.ncell, d_work + R.work_base + L.face_off, L.nface);
     }
     for (int s = 0; s < ns; ++s)
@@ -1637,7 +1645,7 @@ std::function<void()> plan_mixed_batch(const std::vector<std::vector<MixedBlock>
                                 std::to_string(L.nitems) + (L.kpoint ? "/sf_z" : "/sf");
         if (tuned->count(key) || capturing(stream)) continue;
         (*tuned)[key] = time_sf32(stream, [&]() {
-          sf_launch32(stream, sm, L.mesh, L.kpoint, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
+          sf_launch32(stream, sm, L.mesh, L.kpoint, L.width, sf::Item<float>{}, d_sf + R.sf_base + L.item_off,
                       d_work + R.work_base + L.cell_off, L.ncell, d_work + R.work_base + L.face_off, L.nface);
         });
       }
@@ -1995,6 +2003,11 @@ static bool apply_df_tiled(dftfe_ham h, const double* X, int64_t ldx, double* Y,
 
 // Y = H~ X with the pair-of-floats cell products (nonlocal part FP64).
 void apply_df(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, bool with_nl) {
+  if (sf_applicable(h->mesh)) {
+    sf_local_pairs(h, X, ldx, Y, ldy, ncol, nullptr);
+    if (with_nl) nonlocal_add_fp64(h, X, ldx, Y, ldy, ncol, 1.0);
+    return;
+  }
   // tiled kernel for the degrees it is instantiated for (rows per thread TM = ceil(nc/32))
   if (apply_df_tiled<1>(h, X, ldx, Y, ldy, ncol, with_nl) || apply_df_tiled<2>(h, X, ldx, Y, ldy, ncol, with_nl) ||
       apply_df_tiled<4>(h, X, ldx, Y, ldy, ncol, with_nl) || apply_df_tiled<7>(h, X, ldx, Y, ldy, ncol, with_nl) ||

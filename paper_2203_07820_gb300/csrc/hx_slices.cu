@@ -527,6 +527,21 @@ bool apply_slices(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t 
   using namespace oz;
   if (!slices_applicable(h)) return false;
   auto* m = h->mesh;
+  if (sf_applicable(m)) {
+    // float pairs through the 1D contractions, each column scaled by its largest entry's power of two:
+    // 48 bits relative to the column where the digits keep 41, no cell matrices to cut or stream (12^3
+    // cells, p = 6, 256 columns: see sf_local_pairs)
+    int* ex = (int*)ws_get(h, "slices_xe", sizeof(int) * (size_t)std::max(ncol, (int)kBlk));
+    DFTFE_CHECK_CUDA(cudaMemsetAsync(ex, 0, sizeof(int) * (size_t)std::max(ncol, (int)kBlk), h->stream));
+    const unsigned gx = (unsigned)std::max(1, h->sm_count) * 4;
+    for (int b0 = 0; b0 < ncol; b0 += kBlk) {
+      ProfScope ps(h, "slices_digits");
+      DFTFE_LAUNCH(k_col_exponent, gx, 256, 0, h->stream, X + b0, ldx, m->M, std::min((int)kBlk, ncol - b0), ex + b0);
+    }
+    sf_local_pairs(h, X, ldx, Y, ldy, ncol, ex);
+    if (with_nl) nonlocal_add_fp64(h, X, ldx, Y, ldy, ncol, 1.0);
+    return true;
+  }
   const int nc = m->nc;
   const int nmt = (nc + 127) / 128;
   const int rows8 = ((nc - 128 * (nmt - 1)) + 7) / 8 * 8;
@@ -580,10 +595,12 @@ bool apply_slices(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t 
   return true;
 }
 
-// W = H~X for the mixed Rayleigh-Ritz step: exact digit products where they apply, else the
-// float-pair products
+// W = H~X for the mixed Rayleigh-Ritz step: float pairs through the 1D contractions (the columns are
+// orthonormal: no scaling), or on dense cell products exact digit products, beyond their degrees
+// float pairs
 void apply_w(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, bool with_nl) {
-  if (!apply_slices(h, X, ldx, Y, ldy, ncol, with_nl)) apply_df(h, X, ldx, Y, ldy, ncol, with_nl);
+  if (sf_applicable(h->mesh)) apply_df(h, X, ldx, Y, ldy, ncol, with_nl);
+  else if (!apply_slices(h, X, ldx, Y, ldy, ncol, with_nl)) apply_df(h, X, ldx, Y, ldy, ncol, with_nl);
 }
 
 }  // namespace dftfe

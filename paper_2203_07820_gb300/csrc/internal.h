@@ -7,6 +7,8 @@
 #include <string>
 #include <vector>
 #include <map>
+#include <memory>
+#include <mutex>
 #include <stdexcept>
 #include <atomic>
 #include <functional>
@@ -80,6 +82,9 @@ struct dftfe_mesh_s {
   std::vector<double> D;      // n1 x n1 derivative matrix at GLL nodes
   std::vector<double> Lq;     // nq1 x n1: l_a at the potential quadrature points
   std::vector<double> m1[3];  // 1D lumped mass per axis
+  // tables of the tensor-product kernels, formed on first use (sumfac.cu)
+  mutable std::mutex sf_mutex;
+  mutable std::shared_ptr<void> sf_tables[3];
 };
 
 namespace dftfe {
@@ -159,6 +164,7 @@ struct dftfe_ham_s {
   int64_t mixed_version[2] = {-1, -1};  // potential version of the split tiles (bf16, tf32)
   int64_t df_version = -1;              // potential version of the float-pair cell matrices
   int64_t sf32_version = -1;            // potential version of the FP32 scaled potential
+  int64_t sfdf_version = -1;            // potential version of its float pairs
   int64_t slices_version = -1;          // potential version of the digit rows (exact slices)
   // a3: nonlocal (CSR by projector and by node)
   int nproj = 0;
@@ -273,11 +279,13 @@ void sf_launch64(cudaStream_t s, int sm, const dftfe_mesh_s* m, const sf::Item<d
 const float* sf_potential32(dftfe_ham h);
 sf::Item<float> sf_item32(dftfe_ham h, const float* v, float* face, const float* X, int64_t ldx, const float* Xp,
                           int64_t ldp, float* Z, int64_t ldz, int ncol, double alpha, double s1, double s2);
-int64_t sf_cell_work32(const dftfe_mesh_s* m, int ncol);
-void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, const sf::Item<float>& one,
+int64_t sf_cell_work32(const dftfe_mesh_s* m, int ncol, int width);
+int sf_width32(int sm, int n1, int64_t items4);      // columns per thread (2 or 4) from the items of width 4
+void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, int width, const sf::Item<float>& one,
                  const sf::Item<float>* items, const int2* cell_work, int64_t ncell_work, const int2* face_work,
                  int64_t nface_work);
 
+void sf_local_pairs(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, const int* ex);
 void sf_density(dftfe_ham h, const double* Xo, int64_t ldo, int ncol, const double* Xfr, int64_t ldf, int nfr,
                 const double* f_fr, double* rho);
 
@@ -362,7 +370,6 @@ void tri_inverse_blocked(dftfe_ham h, double* L, double* Z, int N);
 void rotate_inplace(dftfe_ham h, double* X, int64_t ld, int64_t M, int N, const double* Z,
                     bool upper);
 void syevd(dftfe_ham h, double* A, int N, double* evals, double* Q, int* d_status);
-void tridiag_ql(cudaStream_t s, double* d, double* e, double* Z, int N, int* d_status);
 // cw = 2: complex columns (interleaved real and imaginary parts, ld in doubles), one
 // residual per complex column
 void residual_norms(dftfe_ham h, const double* X, int64_t ldx, const double* W, int64_t ldw,

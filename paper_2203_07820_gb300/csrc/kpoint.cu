@@ -449,14 +449,15 @@ void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ld
   }
 }
 
-// W = H~^k X with an FP64-accurate local part on the real view (prec: DFTFE_FP64_SLICES, the
-// exact digit products, or DFTFE_FP64_FLOAT_PAIRS) and the k-dependent and nonlocal terms in
-// FP64: the W of a mixed complex Rayleigh-Ritz
+// W = H~^k X with an FP64-accurate local part on the real view (prec: DFTFE_FP64_SLICES or
+// DFTFE_FP64_FLOAT_PAIRS; w: the form of the mixed Rayleigh-Ritz) and the k-dependent and nonlocal
+// terms in FP64
 static void apply_z_df(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol,
-                       dftfe_precision prec) {
+                       dftfe_precision prec, bool w = false) {
   require_kpoint(h);
   auto* m = h->mesh;
-  if (prec == DFTFE_FP64_SLICES) apply_w(h, X, 2 * ldx, Y, 2 * ldy, 2 * ncol, false);
+  if (w) apply_w(h, X, 2 * ldx, Y, 2 * ldy, 2 * ncol, false);
+  else if (prec == DFTFE_FP64_SLICES) apply_slices(h, X, 2 * ldx, Y, 2 * ldy, 2 * ncol, false);
   else apply_df(h, X, 2 * ldx, Y, 2 * ldy, 2 * ncol, false);
   const double k2 = h->kvec[0] * h->kvec[0] + h->kvec[1] * h->kvec[1] + h->kvec[2] * h->kvec[2];
   const int p = m->p;
@@ -553,7 +554,7 @@ static void rayleigh_ritz_z(dftfe_ham h, double* X, int64_t ld, int ncol, double
   auto* m = h->mesh;
   const int N2 = 2 * ncol;
   // W FP64-accurate in both precisions (float pairs for the local part of a mixed pass)
-  if (mixed) apply_z_df(h, X, ld, W, ldw, ncol, DFTFE_FP64_SLICES);
+  if (mixed) apply_z_df(h, X, ld, W, ldw, ncol, DFTFE_FP64_SLICES, true);
   else apply_combo_z(h, X, ld, nullptr, 0, W, ldw, ncol, 1.0, 0.0, 0.0);
   double* G = (double*)ws_get(h, "Hhat", sizeof(double) * (size_t)N2 * N2);
   real_view_gram(h, X, 2 * ld, W, 2 * ldw, N2, G, mixed);

@@ -2,8 +2,12 @@
 // shared faces, and their launches for one system and for the batched passes.
 #include "internal.h"
 #include "sumfac.h"
+#include "tcgen05.h"
 
 #include <algorithm>
+#include <memory>
+#include <mutex>
+#include <type_traits>
 #include <cmath>
 #include <vector>
 
@@ -21,6 +25,18 @@ __device__ __forceinline__ int load_item(sf::Item<T>& it, const sf::Item<T>& one
   return wk.y;
 }
 
+// FP64 -> float pair with the narrowing and widening as integer operations (one FP64 subtraction)
+__device__ __forceinline__ sf::DF to_pair(double x) {
+  const float hi = tc::narrow_f64(x);
+  return sf::DF{hi, tc::narrow_f64(x - tc::widen_f32(hi))};
+}
+// For a column whose largest entry has biased exponent e (0: an all-zero column): 2^(e - 1022), its
+// scale, or with -e the reciprocal (the ends of the range drawn in, so that both are normal numbers).
+__device__ __forceinline__ double scale_of(int e) {
+  const int m = min(max(abs(e), 2), 2044);
+  return __longlong_as_double((long long)(e > 0 ? m + 1 : e < 0 ? 2045 - m : 1023) << 52);
+}
+
 // Where a work item lies: slots of one cell per CTA, columns of slots per row of cells, the first
 // cell and its mesh position, the first slot column.  (The divisions of every thread otherwise.)
 struct SfPlace {
@@ -28,7 +44,7 @@ struct SfPlace {
 };
 template <typename T, int CB, int W>
 __device__ __forceinline__ void find_place(const sf::Item<T>& it, int w, int sub, SfPlace& q) {
-  const int nv = (it.ncol + W - 1) / W;
+  const int nv = W ? (it.ncol + W - 1) / (W ? W : 1) : it.ncol;
   int cols = CB;                               // the power of two that holds nv
   while (cols > 1 && cols / 2 >= nv) cols /= 2;
   const int tiles = (nv + cols - 1) / cols;
@@ -42,11 +58,16 @@ __device__ __forceinline__ void find_place(const sf::Item<T>& it, int w, int sub
   q.cy = cyz - q.cz * it.ny;
 }
 
-// eight bytes from global to shared memory, asynchronously (zeros when !ok)
-__device__ __forceinline__ void copy8(void* dst, const void* src, bool ok) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
-               "r"(ok ? 8 : 0)
-               : "memory");
+// eight or sixteen bytes from global to shared memory, asynchronously (zeros when !ok)
+template <typename V> __device__ __forceinline__ void copy_async(V* dst, const void* src, bool ok) {
+  if constexpr (sizeof(V) == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+                 "r"(ok ? 8 : 0)
+                 : "memory");
 }
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int LEFT> __device__ __forceinline__ void copy_wait() {
@@ -72,42 +93,47 @@ template <int LEFT> __device__ __forceinline__ void copy_wait() {
 // has read the last of it, this item's Xp during its first stages, the potential one stage ahead.
 // FP64: bound by the FP64 pipe (2 FMA per clock and SM), about 350 operations per line of seven
 // nodes against 2401 in the dense product.
-template <typename T> struct SfVecOf;
-template <> struct SfVecOf<double> {
-  using V = double;
-  static constexpr int W = 1;
-  __device__ static V zero() { return 0.0; }
-};
-template <> struct SfVecOf<float> {
-  using V = sf::F2;
-  static constexpr int W = 2;
-  __device__ static V zero() { return {0.f, 0.f}; }
-};
+//   W columns per thread and slot: 1 in FP64; 2 in FP32, or 4 (one CTA per SM at p = 6, twice the
+//   independent work per thread, table entries and addresses shared) where it is the faster form
+//   and the items fill the SMs: see quad_pays.
+//   W = 0: FP64 blocks in and out, float pairs inside (Z = H~_loc X alone: alpha = 1, no recurrence).
+template <int W> struct SfVec_;
+template <> struct SfVec_<0> { using V = sf::DF; using C = sf::DF; };
+template <> struct SfVec_<1> { using V = double; using C = double; };
+template <> struct SfVec_<2> { using V = sf::F2; using C = sf::F2; };
+template <> struct SfVec_<4> { using V = sf::F4; using C = sf::F2; };
 
-template <typename T, int N> struct SfCfg {
+template <int W, int N> struct SfCfg {
   static constexpr int CB = N >= 4 ? 8 : (N == 3 ? 16 : 32);
   static constexpr int LINES = N * N;
   static constexpr int THREADS = (LINES * CB + 31) / 32 * 32;
   static constexpr int NP = N == 4 || N == 6 ? N + 1 : N;       // x pitch: odd, so that the x lines of
   static constexpr int NODES = N * N * NP;                       // a warp fall into different banks
   static constexpr int INNER = (N - 2) * (N - 2) * (N - 2);
-  static constexpr int MINB = N == 9 ? 1 : N >= 7 ? 2 : N == 6 ? 3 : N == 5 ? 4 : N == 3 ? 5 : 6;
-  static constexpr size_t smem(bool nodal) { return ((size_t)(nodal ? 2 : 3) * NODES + INNER) * CB * 8; }
+  static constexpr int UB = W == 4 ? 2 : 1;                      // buffers of U
+  static constexpr int MINB = W == 4 ? (N == 7 ? 1 : 2)
+                                     : N == 9 ? 1 : N >= 7 ? 2 : N == 6 ? 3 : N == 5 ? 4 : N == 3 ? 5 : 6;
+  static constexpr size_t smem(bool nodal) {
+    return ((size_t)(nodal ? 1 : 2) * NODES + UB * NODES + INNER) * CB * sizeof(typename SfVec_<W>::V);
+  }
 };
 
-template <typename T, int N, bool NODAL, bool KPT>
-__global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
-    k_sf_cell(const __grid_constant__ sf::Tables<typename SfVecOf<T>::V, N> tab,
-              const __grid_constant__ sf::AntiParity<typename SfVecOf<T>::V, N> G,
+template <typename T, int W, int N, bool NODAL, bool KPT>
+__global__ void __launch_bounds__(SfCfg<W, N>::THREADS, SfCfg<W, N>::MINB)
+    k_sf_cell(const __grid_constant__ sf::Tables<typename SfVec_<W>::C, N> tab,
+              const __grid_constant__ sf::AntiParity<typename SfVec_<W>::C, N> G,
               const __grid_constant__ sf::Item<T> one, const sf::Item<T>* __restrict__ items,
               const int2* __restrict__ work, int nwork) {
-  using Cfg = SfCfg<T, N>;
-  using V = typename SfVecOf<T>::V;
-  constexpr int CB = Cfg::CB, p = N - 1, W = SfVecOf<T>::W;
-  const V vzero = SfVecOf<T>::zero();
+  using Cfg = SfCfg<W, N>;
+  using V = typename SfVec_<W>::V;
+  using C = typename SfVec_<W>::C;
+  constexpr int CB = Cfg::CB, p = N - 1, UB = Cfg::UB, CW = W ? W : 1;      // columns per slot
+  constexpr bool PAIRS = W == 0;
+  const V vzero = V{};
   extern __shared__ double2 sfsm[];
-  V* const U = reinterpret_cast<V*>(sfsm);
-  V* const R = U + Cfg::NODES * CB;
+  V* U = reinterpret_cast<V*>(sfsm);
+  V* Unext = U + (UB - 1) * Cfg::NODES * CB;
+  V* const R = U + UB * Cfg::NODES * CB;
   V* const P = R + Cfg::NODES * CB;                       // Xp on the interior nodes
   V* const B = P + Cfg::INNER * CB;                       // T
   __shared__ sf::Item<T> its[2];
@@ -145,11 +171,11 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
     int sub = slot;
     if (f.cols < CB) {                         // several cells: each slot its own
       sub = slot % f.cols;
-      find_place<T, CB, W>(it, w, slot / f.cols, f);
+      find_place<T, CB, CW>(it, w, slot / f.cols, f);
     }
     Place q;
     q.cell = f.cell;
-    q.col = (f.vcol + sub) * W;
+    q.col = (f.vcol + sub) * CW;
     q.ok = on && f.cz < it.nz && q.col < it.ncol;
     int iy = f.cy * p + i, iz = f.cz * p + j;
     iy = iy == it.ny * p ? 0 : iy;
@@ -158,57 +184,94 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
     q.last = f.cx + 1 < it.nx ? p : -f.cx * p;
     return q;
   };
-  auto fetch = [&](const sf::Item<T>& it, const Place& q) {
+  auto fetch = [&](V* U, const sf::Item<T>& it, const Place& q) {
     if (!on) return;
     const T* x = q.ok ? it.X + q.row * it.ldx + q.col : it.X;
 #pragma unroll
     for (int a = 0; a < N; ++a)
-      copy8(&U[xl + a * CB], q.ok ? x + (a < p ? a : q.last) * it.ldx : x, q.ok);
+      copy_async(&U[xl + a * CB], q.ok ? x + (a < p ? a : q.last) * it.ldx : x, q.ok);
   };
   // (Im u, -Re u) of a complex column
   auto turn = [&](V (&x)[N]) {
     if constexpr (KPT) {
 #pragma unroll
-      for (int a = 0; a < N; ++a) x[a] = V{x[a].y, -x[a].x};
+      for (int a = 0; a < N; ++a) {
+        if constexpr (W == 4) x[a] = V{{x[a].a.y, -x[a].a.x}, {x[a].b.y, -x[a].b.x}};
+        else x[a] = V{x[a].y, -x[a].x};
+      }
     }
   };
   __shared__ SfPlace first[2];
   auto load = [&](int buf, int w) {
     const int wl = load_item(its[buf], one, items, work, w);
-    if (threadIdx.x == 0) find_place<T, CB, W>(items ? items[work[w].x] : one, wl, 0, first[buf]);
+    if (threadIdx.x == 0) find_place<T, CB, CW>(items ? items[work[w].x] : one, wl, 0, first[buf]);
     return wl;
   };
   int cur = 0;
   int wloc = load(0, (int)blockIdx.x);
   __syncthreads();
   Place q = place(its[0], first[0], wloc);
-  fetch(its[0], q);
+  fetch(U, its[0], q);
   copy_commit();
   for (int w = blockIdx.x; w < nwork; w += gridDim.x, cur ^= 1) {
     const sf::Item<T>& it = its[cur];
     const bool more = w + (int)gridDim.x < nwork;
     copy_wait<0>();
     __syncthreads();
+    Place next = q;
     if (more) wloc = load(cur ^ 1, w + (int)gridDim.x);
     if (q.ok && inside && it.Xp) {
       const T* xp = it.Xp + q.row * it.ldp + q.col;
 #pragma unroll
-      for (int a = 1; a < p; ++a) copy8(Pl + a * CB, xp + a * it.ldp, true);
+      for (int a = 1; a < p; ++a) copy_async(Pl + a * CB, xp + a * it.ldp, true);
     }
     copy_commit();
-    T vv[N];                                              // the potential of this thread's z line
+    // scalars of the kernel's arithmetic: T, or float pairs (whose potential is stored as pairs)
+    using E = std::conditional_t<PAIRS, sf::DF, T>;
+    E vv[N];                                              // the potential of this thread's z line
     {
-      const T* v = it.v + (int64_t)q.cell * (N * N * N) + (NODAL ? (j * N + i) * N : j * N + i);
+      const E* v = reinterpret_cast<const E*>(it.v) + (int64_t)q.cell * (N * N * N) +
+                   (NODAL ? (j * N + i) * N : j * N + i);
 #pragma unroll
-      for (int c = 0; c < N; ++c) vv[c] = q.ok ? __ldg(v + c * (NODAL ? 1 : N * N)) : T(0);
+      for (int c = 0; c < N; ++c) {
+        vv[c] = E{};
+        if (q.ok) {
+          if constexpr (PAIRS) {
+            const float2 t = __ldg(reinterpret_cast<const float2*>(v + c * (NODAL ? 1 : N * N)));
+            vv[c] = sf::DF{t.x, t.y};
+          } else {
+            vv[c] = __ldg(v + c * (NODAL ? 1 : N * N));
+          }
+        }
+      }
     }
-    V u[N], r[N], k[N], e[(N + 1) / 2], o[N / 2], x0[N];
+    E kyx, kzx, kx;
+    if constexpr (PAIRS) {
+      kyx = to_pair(it.kyx);
+      kzx = to_pair(it.kzx);
+      kx = to_pair(it.kx);
+    } else {
+      kyx = it.kyx;
+      kzx = it.kzx;
+      kx = it.kx;
+    }
+    V u[N], r[N], k[N], e[(N + 1) / 2], o[N / 2], x0[UB == 1 && !PAIRS ? N : 1];
     if (on) {
 #pragma unroll
-      for (int a = 0; a < N; ++a) x0[a] = u[a] = U[xl + a * CB];
+      for (int a = 0; a < N; ++a) {
+        u[a] = U[xl + a * CB];
+        if constexpr (PAIRS) {
+          // the copied FP64 entry, scaled by its column's power of two, becomes a pair
+          double x = __hiloint2double(__float_as_int(u[a].lo), __float_as_int(u[a].hi));
+          if (it.ex) x *= scale_of(-it.ex[q.ok ? q.col : 0]);
+          u[a] = to_pair(x);
+          U[xl + a * CB] = u[a];
+        }
+        if (UB == 1 && !PAIRS) x0[a] = u[a];
+      }
       sf::split<V, N>(u, e, o);
       if (!NODAL) {
-        sf::contract<V, V, N>(tab.L, e, o, r);
+        sf::contract<C, V, N>(tab.L, e, o, r);
 #pragma unroll
         for (int a = 0; a < N; ++a) B[xl + a * CB] = r[a];
       }
@@ -219,16 +282,24 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
         for (int a = 0; a < N; ++a) k[a] = vzero;
       }
       if (NODAL) {     // v u joins the kinetic sums, in their units
-        const T rk = T(1) / it.kx;
+        E rk;
+        if constexpr (PAIRS) rk = to_pair(1.0 / it.kx);
+        else rk = T(1) / it.kx;
 #pragma unroll
         for (int a = 0; a < N; ++a) k[a] = sf::fma(vv[a] * rk, u[a], k[a]);
       }
-      if (KPT && owned) {
-        turn(u);
-        sf::add_anti<V, T, V, N>(G, it.gx, u, k);
+      if constexpr (KPT) {
+        if (owned) {
+          turn(u);
+          sf::add_anti<C, T, V, N>(G, it.gx, u, k);
+        }
       }
     }
-    if (!NODAL) __syncthreads();
+    __syncthreads();
+    if (more && UB == 2) {
+      next = place(its[cur ^ 1], first[cur ^ 1], wloc);
+      fetch(Unext, its[cur ^ 1], next);
+    }
     // y line (a = i, ., c = j)
     if (on) {
       if (owned) {
@@ -237,10 +308,10 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
         sf::split<V, N>(u, e, o);
         sf::kinetic<N>(tab.K, u, e, o, r);
 #pragma unroll
-        for (int b = 0; b < N; ++b) r[b] = it.kyx * r[b];
-        if (KPT) {
+        for (int b = 0; b < N; ++b) r[b] = kyx * r[b];
+        if constexpr (KPT) {
           turn(u);
-          sf::add_anti<V, T, V, N>(G, it.gy, u, r);
+          sf::add_anti<C, T, V, N>(G, it.gy, u, r);
         }
 #pragma unroll
         for (int b = 0; b < N; ++b) R[yl + b * SY] = r[b];
@@ -251,7 +322,7 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
       if (!NODAL) {
 #pragma unroll
         for (int b = 0; b < N; ++b) u[b] = B[yl + b * SY];
-        sf::apply<V, V, N>(tab.L, u, r);
+        sf::apply<C, V, N>(tab.L, u, r);
 #pragma unroll
         for (int b = 0; b < N; ++b) B[yl + b * SY] = r[b];
       }
@@ -265,10 +336,10 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
         sf::split<V, N>(u, e, o);
         sf::kinetic<N>(tab.K, u, e, o, r);
 #pragma unroll
-        for (int c = 0; c < N; ++c) r[c] = sf::fma(it.kzx, r[c], R[zl + c * SZ]);
-        if (KPT) {
+        for (int c = 0; c < N; ++c) r[c] = sf::fma(kzx, r[c], R[zl + c * SZ]);
+        if constexpr (KPT) {
           turn(u);
-          sf::add_anti<V, T, V, N>(G, it.gz, u, r);
+          sf::add_anti<C, T, V, N>(G, it.gz, u, r);
         }
 #pragma unroll
         for (int c = 0; c < N; ++c) R[zl + c * SZ] = r[c];
@@ -276,26 +347,25 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
       if (!NODAL) {
 #pragma unroll
         for (int c = 0; c < N; ++c) u[c] = B[zl + c * SZ];
-        sf::apply<V, V, N>(tab.L, u, r);
+        sf::apply<C, V, N>(tab.L, u, r);
 #pragma unroll
         for (int c = 0; c < N; ++c) u[c] = vv[c] * r[c];
-        sf::apply<V, V, N>(tab.Lt, u, r);
+        sf::apply<C, V, N>(tab.Lt, u, r);
 #pragma unroll
         for (int c = 0; c < N; ++c) B[zl + c * SZ] = r[c];
       }
     }
     __syncthreads();
-    Place next = q;
-    if (more) {                                           // U is free: the next item's nodes
+    if (more && UB == 1) {                                // U is free: the next item's nodes
       next = place(its[cur ^ 1], first[cur ^ 1], wloc);
-      fetch(its[cur ^ 1], next);
+      fetch(U, its[cur ^ 1], next);
     }
     copy_commit();
     if (!NODAL) {
       if (on) {
 #pragma unroll
         for (int b = 0; b < N; ++b) u[b] = B[yl + b * SY];
-        sf::apply<V, V, N>(tab.Lt, u, r);
+        sf::apply<C, V, N>(tab.Lt, u, r);
 #pragma unroll
         for (int b = 0; b < N; ++b) B[yl + b * SY] = r[b];
       }
@@ -304,16 +374,26 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
     if (q.ok) {
       if (NODAL) {
 #pragma unroll
-        for (int a = 0; a < N; ++a) r[a] = it.kx * (k[a] + R[xl + a * CB]);
+        for (int a = 0; a < N; ++a) r[a] = kx * (k[a] + R[xl + a * CB]);
       } else {
 #pragma unroll
         for (int a = 0; a < N; ++a) u[a] = B[xl + a * CB];
-        sf::apply<V, V, N>(tab.Lt, u, r);
+        sf::apply<C, V, N>(tab.Lt, u, r);
 #pragma unroll
-        for (int a = 0; a < N; ++a) r[a] = sf::fma(it.kx, k[a] + R[xl + a * CB], r[a]);
+        for (int a = 0; a < N; ++a) r[a] = sf::fma(kx, k[a] + R[xl + a * CB], r[a]);
       }
       T* const face = it.face + ((int64_t)q.cell * sf::surface_count<N>() + fline) * it.ldf + q.col;
-      if (!inside) {
+      if constexpr (PAIRS) {
+        const double sc = it.ex ? scale_of(it.ex[q.col]) : 1.0;
+        T* z = it.Z + q.row * it.ldz + q.col;
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+          const double y = (tc::widen_f32(r[a].hi) + tc::widen_f32(r[a].lo)) * sc;
+          if (!inside) face[a * it.ldf] = y;
+          else if (a == 0 || a == p) face[a ? it.ldf : 0] = y;
+          else z[a * it.ldz] = y;
+        }
+      } else if (!inside) {
 #pragma unroll
         for (int a = 0; a < N; ++a) *reinterpret_cast<V*>(face + a * it.ldf) = r[a];
       } else {
@@ -321,15 +401,22 @@ __global__ void __launch_bounds__(SfCfg<T, N>::THREADS, SfCfg<T, N>::MINB)
         *reinterpret_cast<V*>(face + it.ldf) = r[p];
         T* z = it.Z + q.row * it.ldz + q.col;
         const bool xp = it.Xp != nullptr;
-        copy_wait<1>();                                   // this thread's own Xp
+        if (UB == 1) copy_wait<1>();                      // this thread's own Xp
+        else if (more) copy_wait<1>();
+        else copy_wait<0>();
 #pragma unroll
         for (int a = 1; a < p; ++a) {
           const V y = xp ? sf::fma(it.alpha, r[a], it.s2 * Pl[a * CB]) : it.alpha * r[a];
-          *reinterpret_cast<V*>(z + a * it.ldz) = sf::fma(it.s1, x0[a], y);
+          *reinterpret_cast<V*>(z + a * it.ldz) = sf::fma(it.s1, UB == 1 ? x0[a] : U[xl + a * CB], y);
         }
       }
     }
     q = next;
+    if (UB == 2) {
+      V* t = U;
+      U = Unext;
+      Unext = t;
+    }
   }
 }
 
@@ -421,8 +508,8 @@ __global__ void k_sf_narrow(const double* __restrict__ v, int64_t n, float* __re
 // copy of rho (k_sf_density_sum adds the copies in order).  Bound by the FP64 pipe: 125
 // operations per line of seven nodes and column against 2401 in the dense interpolation.
 template <int N> struct SfDen {
-  static constexpr int CB = SfCfg<double, N>::CB, THREADS = SfCfg<double, N>::THREADS;
-  static constexpr int NODES = SfCfg<double, N>::NODES;
+  static constexpr int CB = SfCfg<1, N>::CB, THREADS = SfCfg<1, N>::THREADS;
+  static constexpr int NODES = SfCfg<1, N>::NODES;
   static constexpr int MINB = N == 9 ? 1 : N >= 7 ? 2 : 3;
   static constexpr size_t smem() { return (size_t)2 * NODES * CB * sizeof(double); }
 };
@@ -431,7 +518,7 @@ __global__ void __launch_bounds__(SfDen<N>::THREADS, SfDen<N>::MINB)
     k_sf_density(const __grid_constant__ sf::Parity<double, N> L, int nx, int ny, int nz,
                  const double* __restrict__ Xo, int64_t ldo, int ncol, const double* __restrict__ Xfr, int64_t ldf,
                  int nfr, const double* __restrict__ f_fr, double scale, double* __restrict__ rho, int64_t copy) {
-  constexpr int CB = SfDen<N>::CB, p = N - 1, NP = SfCfg<double, N>::NP, SY = NP * CB, SZ = N * NP * CB;
+  constexpr int CB = SfDen<N>::CB, p = N - 1, NP = SfCfg<1, N>::NP, SY = NP * CB, SZ = N * NP * CB;
   extern __shared__ double2 sfdn[];
   double* B = reinterpret_cast<double*>(sfdn);
   double* B2 = B + SfDen<N>::NODES * CB;
@@ -547,8 +634,8 @@ template <typename T, int N> static sf::Parity<T, N> parity(const std::vector<do
   return r;
 }
 
-template <int N> static void kinetic_table(const dftfe_mesh_s* m, sf::Parity<double, N>& K) {
-  K = parity<double, N>(kinetic1d(m));
+template <int N, typename C> static void kinetic_table(const dftfe_mesh_s* m, sf::Parity<C, N>& K) {
+  K = parity<C, N>(kinetic1d(m));
 }
 template <int N> static void kinetic_table(const dftfe_mesh_s* m, sf::Differences<sf::F2, N>& D) {
   const std::vector<double> K = kinetic1d(m), wa = assembled_weights(m);
@@ -630,7 +717,7 @@ static sf::Item<T> make_item(dftfe_ham h, const T* v, T* face, const T* X, int64
   return sf::Item<T>{v, X, Xp, Z, face, ldx, ldp, ldz, ncol, face_ld(ncol), m->n[0], m->n[1], m->n[2],
                      (T)kx, (T)(ky / kx), (T)(kz / kx), (T)(h->kvec[0] * (2.0 / m->h[0]) / kx),
                      (T)(h->kvec[1] * (2.0 / m->h[1]) / kx), (T)(h->kvec[2] * (2.0 / m->h[2]) / kx), (T)alpha,
-                     (T)s1, (T)s2};
+                     (T)s1, (T)s2, nullptr};
 }
 
 sf::Item<double> sf_item64(dftfe_ham h, double* face, const double* X, int64_t ldx, const double* Xp, int64_t ldp,
@@ -638,10 +725,10 @@ sf::Item<double> sf_item64(dftfe_ham h, double* face, const double* X, int64_t l
   return make_item<double>(h, loc(h)->d_sfv, face, X, ldx, Xp, ldp, Z, ldz, ncol, alpha, s1, s2);
 }
 
-// CTAs of the cell kernel for one system
-template <typename T, int N> static int64_t cell_work(const dftfe_mesh_s* m, int ncol) {
-  constexpr int CB = SfCfg<T, N>::CB, W = SfVecOf<T>::W;
-  const int nv = (ncol + W - 1) / W;
+// work items of the cell kernel for one system
+template <int W, int N> static int64_t cell_work(const dftfe_mesh_s* m, int ncol) {
+  constexpr int CB = SfCfg<W, N>::CB, CW = W ? W : 1;
+  const int nv = (ncol + CW - 1) / CW;
   int cols = CB;
   while (cols > 1 && cols / 2 >= nv) cols /= 2;
   return ((m->Nc + CB / cols - 1) / (CB / cols)) * ((nv + cols - 1) / cols);
@@ -676,6 +763,11 @@ template <typename T, int N> static sf::AntiParity<T, N> anti_table(const dftfe_
   return r;
 }
 
+__global__ void k_sf_pairs(const double* __restrict__ v, int64_t n, sf::DF* __restrict__ out) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t < n) out[t] = to_pair(v[t]);
+}
+
 // the FP32 copy of the scaled potential (once per potential, in the owner of the operator)
 const float* sf_potential32(dftfe_ham h) {
   dftfe_ham o = loc(h);
@@ -695,59 +787,92 @@ sf::Item<float> sf_item32(dftfe_ham h, const float* v, float* face, const float*
 
 int64_t sf_cell_work64(const dftfe_mesh_s* m, int ncol) {
   int64_t n = 0;
-  with_n(m->n1, [&](auto k) { n = cell_work<double, decltype(k)::value>(m, ncol); });
+  with_n(m->n1, [&](auto k) { n = cell_work<1, decltype(k)::value>(m, ncol); });
   return n;
 }
-int64_t sf_cell_work32(const dftfe_mesh_s* m, int ncol) {
+int64_t sf_cell_work32(const dftfe_mesh_s* m, int ncol, int width) {
   int64_t n = 0;
-  with_n(m->n1, [&](auto k) { n = cell_work<float, decltype(k)::value>(m, ncol); });
+  with_n(m->n1, [&](auto k) {
+    constexpr int N = decltype(k)::value;
+    n = width == 4 ? cell_work<4, N>(m, ncol) : cell_work<2, N>(m, ncol);
+  });
   return n;
+}
+// Columns per thread of the FP32 kernel (both widths give the same bits).  Four at p = 4 and 6, where
+// they measured 10 to 12 % faster over 128 columns (12^3 cells, p = 6: 289 against 323 us a launch;
+// 14^3, p = 4: 7 % of the filter), once there are eight items per resident CTA; with fewer the last
+// wave costs more (8^3 cells, p = 6, 37 columns: 47 against 40 us).  p = 5 measured the same.
+int sf_width32(int sm, int n1, int64_t items4) {
+  return (n1 == 5 || n1 == 7) && items4 >= 8LL * sm * (n1 == 7 ? 1 : 2) ? 4 : 2;
 }
 
-template <typename T, int N, bool NODAL, bool KPT>
-static void launch_cell(cudaStream_t s, int sm, const sf::Tables<typename SfVecOf<T>::V, N>& tab,
-                        const sf::AntiParity<typename SfVecOf<T>::V, N>& G, const sf::Item<T>& one,
+template <typename T, int W, int N, bool NODAL, bool KPT>
+static void launch_cell(cudaStream_t s, int sm, const sf::Tables<typename SfVec_<W>::C, N>& tab,
+                        const sf::AntiParity<typename SfVec_<W>::C, N>& G, const sf::Item<T>& one,
                         const sf::Item<T>* items, const int2* work, int64_t n) {
-  using Cfg = SfCfg<T, N>;
+  using Cfg = SfCfg<W, N>;
   if (n <= 0) return;
   DFTFE_REQUIRE(n < INT32_MAX / 2, "too many (cell, column tile) items for one launch");
-  DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_sf_cell<T, N, NODAL, KPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)Cfg::smem(NODAL)));
+  static const cudaError_t attr = cudaFuncSetAttribute(k_sf_cell<T, W, N, NODAL, KPT>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem(NODAL));
+  DFTFE_CHECK_CUDA(attr);
   // FP32: as many CTAs as stay resident, each walking its items with the next one's nodes in
   // flight; FP64: one CTA per item, since the FP64 pipe hides the loads and a fixed deal of long
   // items would leave it idle at the end
-  const unsigned grid = (unsigned)(sizeof(T) == 8 ? n : std::min<int64_t>(n, (int64_t)sm * Cfg::MINB));
-  DFTFE_LAUNCH((k_sf_cell<T, N, NODAL, KPT>), grid, Cfg::THREADS, Cfg::smem(NODAL), s, tab, G, one, items, work,
+  const unsigned grid = (unsigned)(W <= 1 ? n : std::min<int64_t>(n, (int64_t)sm * Cfg::MINB));
+  DFTFE_LAUNCH((k_sf_cell<T, W, N, NODAL, KPT>), grid, Cfg::THREADS, Cfg::smem(NODAL), s, tab, G, one, items, work,
                (int)n);
 }
 
-void sf_launch64(cudaStream_t s, int sm, const dftfe_mesh_s* m, const sf::Item<double>& one, const sf::Item<double>* items,
-                 const int2* cell_work, int64_t ncell_work, const int2* face_work, int64_t nface_work) {
+// 1D tables of a degree and quadrature rule, formed once per mesh (they depend on neither the box
+// nor the potential)
+template <typename C, int N> struct Tables1D {
+  sf::Tables<C, N> tab;
+  sf::AntiParity<C, N> G;
+};
+template <typename C, int N> static const Tables1D<C, N>& mesh_tables(const dftfe_mesh_s* m) {
+  std::shared_ptr<void>& slot = m->sf_tables[std::is_same<C, double>::value ? 0 : std::is_same<C, sf::F2>::value ? 1 : 2];
+  std::lock_guard<std::mutex> lock(m->sf_mutex);
+  if (!slot) slot = std::make_shared<Tables1D<C, N>>(Tables1D<C, N>{tables<C, N>(m), anti_table<C, N>(m)});
+  return *static_cast<const Tables1D<C, N>*>(slot.get());
+}
+
+void sf_launch64(cudaStream_t s, int sm, const dftfe_mesh_s* m, const sf::Item<double>& one,
+                 const sf::Item<double>* items, const int2* cell_work, int64_t ncell_work, const int2* face_work,
+                 int64_t nface_work) {
   with_n(m->n1, [&](auto k) {
     constexpr int N = decltype(k)::value;
-    const auto tab = tables<double, N>(m);
-    const auto G = anti_table<double, N>(m);
-    if (m->vquad == 1) launch_cell<double, N, true, false>(s, sm, tab, G, one, items, cell_work, ncell_work);
-    else launch_cell<double, N, false, false>(s, sm, tab, G, one, items, cell_work, ncell_work);
+    const auto& t = mesh_tables<double, N>(m);
+    if (m->vquad == 1) launch_cell<double, 1, N, true, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
+    else launch_cell<double, 1, N, false, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
     DFTFE_LAUNCH((k_sf_faces<double, N, 1>), (unsigned)nface_work, 256, 0, s, one, items, face_work);
   });
 }
 
 // kpoint: complex columns (all items of a launch alike); rows of every buffer of a multiple of 4
-// floats, 16-byte aligned, with the columns padded to a multiple of 4
-void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, const sf::Item<float>& one,
+// floats, 16-byte aligned, with the columns padded to a multiple of 4; width: sf_width32 (the cell
+// work list is that of the width)
+void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, int width, const sf::Item<float>& one,
                  const sf::Item<float>* items, const int2* cell_work, int64_t ncell_work, const int2* face_work,
                  int64_t nface_work) {
   with_n(m->n1, [&](auto k) {
     constexpr int N = decltype(k)::value;
     if constexpr (N <= 8) {      // split precision: at most 512 nodes per cell
-      const auto tab = tables<sf::F2, N>(m);
-      const auto G = anti_table<sf::F2, N>(m);
+      const auto& t = mesh_tables<sf::F2, N>(m);
       const bool nodal = m->vquad == 1;
-      if (nodal && kpoint) launch_cell<float, N, true, true>(s, sm, tab, G, one, items, cell_work, ncell_work);
-      else if (nodal) launch_cell<float, N, true, false>(s, sm, tab, G, one, items, cell_work, ncell_work);
-      else if (kpoint) launch_cell<float, N, false, true>(s, sm, tab, G, one, items, cell_work, ncell_work);
-      else launch_cell<float, N, false, false>(s, sm, tab, G, one, items, cell_work, ncell_work);
+      auto cell = [&](auto w) {
+        constexpr int W = decltype(w)::value;
+        if (nodal && kpoint) launch_cell<float, W, N, true, true>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
+        else if (nodal) launch_cell<float, W, N, true, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
+        else if (kpoint) launch_cell<float, W, N, false, true>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
+        else launch_cell<float, W, N, false, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
+      };
+      if constexpr (N == 5 || N == 7) {
+        if (width == 4) cell(std::integral_constant<int, 4>());
+        else cell(std::integral_constant<int, 2>());
+      } else {
+        cell(std::integral_constant<int, 2>());
+      }
       DFTFE_LAUNCH((k_sf_faces<float, N, 4>), (unsigned)nface_work, 256, 0, s, one, items, face_work);
     }
   });
@@ -768,6 +893,37 @@ void sf_local64(dftfe_ham h, const double* X, int64_t ldx, const double* Xp, int
   }
 }
 
+// Y = H~_loc X from float pairs (FP64 blocks; about 2^-44 |H~||X|); ex: biased exponents of the columns'
+// largest entries, by which they are scaled on the way (NULL: the entries lie well inside FP32's range)
+void sf_local_pairs(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, const int* ex) {
+  auto* m = h->mesh;
+  dftfe_ham o = loc(h);
+  const int64_t nvq = m->Nc * m->nq;
+  sf::DF* v = (sf::DF*)ws_get(o, "sf_vdf", sizeof(sf::DF) * nvq);
+  if (o->sfdf_version != o->potential_version) {
+    DFTFE_LAUNCH(k_sf_pairs, (unsigned)((nvq + 255) / 256), 256, 0, h->stream, o->d_sfv, nvq, v);
+    o->sfdf_version = o->potential_version;
+  }
+  double* face = (double*)ws_get(h, "sf_face", sizeof(double) * sf_face_elems(m, std::min(ncol, kSfCols)));
+  for (int c0 = 0; c0 < ncol; c0 += kSfCols) {
+    const int nb = std::min(kSfCols, ncol - c0);
+    sf::Item<double> one = make_item<double>(h, (const double*)v, face, X + c0, ldx, (const double*)nullptr, 0, Y + c0, ldy,
+                                             nb, 1.0, 0.0, 0.0);
+    one.ex = ex ? ex + c0 : nullptr;
+    ProfScope ps(h, "cell_gemm_df");
+    with_n(m->n1, [&](auto k) {
+      constexpr int N = decltype(k)::value;
+      const auto& t = mesh_tables<sf::DF, N>(m);
+      const int64_t n = cell_work<0, N>(m, nb);
+      if (m->vquad == 1)
+        launch_cell<double, 0, N, true, false>(h->stream, h->sm_count, t.tab, t.G, one, nullptr, nullptr, n);
+      else
+        launch_cell<double, 0, N, false, false>(h->stream, h->sm_count, t.tab, t.G, one, nullptr, nullptr, n);
+      DFTFE_LAUNCH((k_sf_faces<double, N, 1>), (unsigned)m->Nc, 256, 0, h->stream, one, nullptr, nullptr);
+    });
+  }
+}
+
 // the density of sf_applicable meshes
 void sf_density(dftfe_ham h, const double* Xo, int64_t ldo, int ncol, const double* Xfr, int64_t ldf, int nfr,
                 const double* f_fr, double* rho) {
@@ -777,14 +933,15 @@ void sf_density(dftfe_ham h, const double* Xo, int64_t ldo, int ncol, const doub
   with_n(m->n1, [&](auto k) {
     constexpr int N = decltype(k)::value;
     using D = SfDen<N>;
-    DFTFE_CHECK_CUDA(cudaFuncSetAttribute(k_sf_density<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)D::smem()));
+    static const cudaError_t attr = cudaFuncSetAttribute(k_sf_density<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         (int)D::smem());
+    DFTFE_CHECK_CUDA(attr);
     // few cells: several CTAs per cell, up to one per column tile, so that every SM has a share
     const int64_t tiles = (ncol + nfr + D::CB - 1) / D::CB;
     const int copies = (int)std::max<int64_t>(1, std::min<int64_t>({tiles, 8, 4LL * D::MINB * h->sm_count / m->Nc}));
     double* part = copies > 1 ? (double*)ws_get(h, "sf_rho", sizeof(double) * n * copies) : rho;
     DFTFE_LAUNCH((k_sf_density<N>), dim3((unsigned)m->Nc, (unsigned)copies), D::THREADS, D::smem(), h->stream,
-                 tables<double, N>(m).L, m->n[0], m->n[1], m->n[2], Xo, ldo, ncol, Xfr, ldf, nfr, f_fr, scale, part, n);
+                 mesh_tables<double, N>(m).tab.L, m->n[0], m->n[1], m->n[2], Xo, ldo, ncol, Xfr, ldf, nfr, f_fr, scale, part, n);
     if (copies > 1)
       DFTFE_LAUNCH(k_sf_density_sum, (unsigned)((n + 255) / 256), 256, 0, h->stream, part, copies, n, rho);
   });

@@ -28,6 +28,17 @@ namespace sf {
 struct alignas(8) F2 {
   float x, y;
 };
+struct alignas(16) F4 {
+  F2 a, b;
+};
+// an unevaluated sum of two floats (about 48 bits), for FP64-accurate products on the FP32 pipes
+struct alignas(8) DF {
+  float hi, lo;
+};
+inline void set(DF& c, double v) {
+  c.hi = (float)v;
+  c.lo = (float)(v - (double)c.hi);
+}
 inline void set(double& c, double v) { c = v; }
 inline void set(F2& c, double v) { c.x = c.y = (float)v; }
 
@@ -81,6 +92,7 @@ template <typename T> struct Item {
   T kx, kyx, kzx;               // kappa_x, kappa_y / kappa_x, kappa_z / kappa_x
   T gx, gy, gz;                 // k_d (2/h_d) / kappa_x (complex columns at a Bloch k-point)
   T alpha, s1, s2;
+  const int* ex;                // float-pair form: biased exponents of the columns (or null)
 };
 
 #ifdef __CUDACC__
@@ -112,7 +124,37 @@ __device__ __forceinline__ F2 operator*(F2 a, F2 b) {
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma(F2{-1.f, -1.f}, b, a); }
 __device__ __forceinline__ F2 fma(float a, F2 b, F2 c) { return fma(F2{a, a}, b, c); }
 __device__ __forceinline__ F2 operator*(float a, F2 b) { return F2{a, a} * b; }
+// four columns
+__device__ __forceinline__ F4 operator+(F4 a, F4 b) { return {a.a + b.a, a.b + b.b}; }
+__device__ __forceinline__ F4 operator-(F4 a, F4 b) { return {a.a - b.a, a.b - b.b}; }
+__device__ __forceinline__ F4 operator*(F2 c, F4 v) { return {c * v.a, c * v.b}; }
+__device__ __forceinline__ F4 operator*(float c, F4 v) { return {c * v.a, c * v.b}; }
+__device__ __forceinline__ F4 fma(F2 c, F4 v, F4 w) { return {fma(c, v.a, w.a), fma(c, v.b, w.b)}; }
+__device__ __forceinline__ F4 fma(float c, F4 v, F4 w) { return {fma(c, v.a, w.a), fma(c, v.b, w.b)}; }
 __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
+// Float pairs: exact products (one FMA for the rounding error) plus the cross terms, Knuth's TwoSum for
+// the leading parts.  The intrinsics keep the compiler from contracting them.
+__device__ __forceinline__ DF two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ DF tidy(DF a) {            // |lo| <= half an ulp of hi
+  const float s = __fadd_rn(a.hi, a.lo);
+  return {s, __fsub_rn(a.lo, __fsub_rn(s, a.hi))};
+}
+__device__ __forceinline__ DF operator*(DF a, DF b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  return {p, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ DF fma(DF a, DF b, DF c) {
+  const DF p = a * b, s = two_sum(c.hi, p.hi);
+  return {s.hi, __fadd_rn(__fadd_rn(c.lo, p.lo), s.lo)};
+}
+__device__ __forceinline__ DF operator+(DF a, DF b) {
+  const DF s = two_sum(a.hi, b.hi);
+  return tidy(DF{s.hi, __fadd_rn(__fadd_rn(a.lo, b.lo), s.lo)});
+}
+__device__ __forceinline__ DF operator-(DF a, DF b) { return a + DF{-b.hi, -b.lo}; }
 
 // T: table entry, V: the thread's columns (both double, or both F2)
 template <typename V, int N>
@@ -155,14 +197,14 @@ __device__ __forceinline__ void apply(const Parity<T, N>& A, const V (&u)[N], V 
 }
 
 // out = K u (e, o: the parity parts of u, formed by the caller; the difference form needs u alone)
-template <int N>
-__device__ __forceinline__ void kinetic(const Parity<double, N>& K, const double (&)[N], const double (&e)[(N + 1) / 2],
-                                        const double (&o)[N / 2], double (&out)[N]) {
-  contract<double, double, N>(K, e, o, out);
+template <int N, typename V>
+__device__ __forceinline__ void kinetic(const Parity<V, N>& K, const V (&)[N], const V (&e)[(N + 1) / 2],
+                                        const V (&o)[N / 2], V (&out)[N]) {
+  contract<V, V, N>(K, e, o, out);
 }
-template <int N>
-__device__ __forceinline__ void kinetic(const Differences<F2, N>& K, const F2 (&u)[N], const F2 (&)[(N + 1) / 2],
-                                        const F2 (&)[N / 2], F2 (&out)[N]) {
+template <int N, typename V>
+__device__ __forceinline__ void kinetic(const Differences<F2, N>& K, const V (&u)[N], const V (&)[(N + 1) / 2],
+                                        const V (&)[N / 2], V (&out)[N]) {
   int q = 0;
 #pragma unroll
   for (int i = 0; i < N; ++i) out[i] = K.diag[i] * u[i];
@@ -170,7 +212,7 @@ __device__ __forceinline__ void kinetic(const Differences<F2, N>& K, const F2 (&
   for (int i = 0; i < N; ++i)
 #pragma unroll
     for (int j = i + 1; j < N; ++j, ++q) {
-      const F2 t = fma(K.rho[q], u[i], u[j]);
+      const V t = fma(K.rho[q], u[i], u[j]);
       out[i] = fma(K.ki[q], t, out[i]);
       out[j] = fma(K.kj[q], t, out[j]);
     }
