@@ -58,19 +58,20 @@ __device__ __forceinline__ void slices3(float f, uint32_t& s1, uint32_t& s2, uin
   s3 = tc::tf32_rn_bits(__float_as_uint(r1 - __uint_as_float(s2)));
 }
 
-// the six slice products of one 32-deep chunk into accumulator d (fresh)
+// the six slice products of one 32-deep chunk into accumulator d (fresh), the smallest first: an
+// MMA truncates at the accumulator's size, which stays 2^-11 of the result's until the last four
 __device__ __forceinline__ void chunk_mma(uint32_t d, uint32_t a0, uint32_t b0) {
   const uint32_t id = tc::idesc(2u, 128, 128);
 #pragma unroll
-  for (int ks = 0; ks < 4; ++ks) {
-    const uint32_t o = ks * 32;
-    tc::mma_tf32(d, tc::sdesc(a0 + o), tc::sdesc(b0 + o), id, ks > 0 ? 1u : 0u);
-    tc::mma_tf32(d, tc::sdesc(a0 + o), tc::sdesc(b0 + kTile + o), id, 1u);
-    tc::mma_tf32(d, tc::sdesc(a0 + kTile + o), tc::sdesc(b0 + o), id, 1u);
-    tc::mma_tf32(d, tc::sdesc(a0 + o), tc::sdesc(b0 + 2 * kTile + o), id, 1u);
-    tc::mma_tf32(d, tc::sdesc(a0 + kTile + o), tc::sdesc(b0 + kTile + o), id, 1u);
-    tc::mma_tf32(d, tc::sdesc(a0 + 2 * kTile + o), tc::sdesc(b0 + o), id, 1u);
-  }
+  for (int order = 2; order >= 0; --order)
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      const uint32_t o = ks * 32;
+#pragma unroll
+      for (int sa = 0; sa <= order; ++sa)
+        tc::mma_tf32(d, tc::sdesc(a0 + sa * kTile + o), tc::sdesc(b0 + (order - sa) * kTile + o), id,
+                     order < 2 || ks > 0 || sa > 0 ? 1u : 0u);
+    }
 }
 
 // epilogue: add chunk kc's 32 x 128 accumulator block of this warp's quadrant into acc
