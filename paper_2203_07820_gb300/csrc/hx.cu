@@ -15,6 +15,7 @@
 // The recurrence (Eq. chebyfilter) is fused: the output is initialised to
 // s1 X_k + s2 X_{k-1} and the local and nonlocal parts accumulate alpha H~ X_k on top.
 #include "internal.h"
+#include "nonlocal.cuh"
 #include "cell_fp64.cuh"
 
 #include <cmath>
@@ -45,63 +46,6 @@ __global__ void k_copy_block(const double* __restrict__ src, int64_t lds, double
   int64_t i = t / ncol;
   int j = (int)(t - i * ncol);
   dst[i * ldd + j] = src[i * lds + j];
-}
-
-// P[a][col] = h_a * sum_{e in supp a} C~[e] X[node_e][col], the sum split over each projector's
-// support so that a long support (thousands of entries) is not one chain of dependent loads per
-// warp: CTA (a, s) sums range s (warp w every 8th entry, four in flight, lane = column) into
-// part[a S + s]; k_nl_coef_reduce adds the S ranges in order.
-constexpr int kNlSplits64 = 8;
-__global__ void __launch_bounds__(256) k_nl_coef_part(const double* __restrict__ X, int64_t ldx, int ncol,
-                                                      const int64_t* __restrict__ prow,
-                                                      const int32_t* __restrict__ pnode,
-                                                      const double* __restrict__ pval, double* __restrict__ part) {
-  __shared__ double red[8][32];
-  const int a = blockIdx.x / kNlSplits64, sidx = blockIdx.x % kNlSplits64;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col = blockIdx.y * 32 + lane;
-  const int64_t e0 = prow[a], e1 = prow[a + 1], len = (e1 - e0 + kNlSplits64 - 1) / kNlSplits64;
-  const int64_t s0 = e0 + sidx * len, s1 = min(e1, s0 + len);
-  double s = 0.0;
-  if (col < ncol) {
-#pragma unroll 4
-    for (int64_t e = s0 + warp; e < s1; e += 8) s = fma(pval[e], X[(int64_t)pnode[e] * ldx + col], s);
-  }
-  red[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0 && col < ncol) {
-    double t = 0.0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) t += red[w][lane];
-    part[(int64_t)blockIdx.x * ncol + col] = t;
-  }
-}
-
-__global__ void k_nl_coef_reduce(const double* __restrict__ part, const double* __restrict__ hcoup, int nproj,
-                                 int ncol, double* __restrict__ P) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nproj * ncol) return;
-  const int64_t a = t / ncol;
-  const int col = (int)(t - a * ncol);
-  double s = 0.0;
-  for (int k = 0; k < kNlSplits64; ++k) s += part[(a * kNlSplits64 + k) * ncol + col];
-  P[t] = hcoup[a] * s;
-}
-
-// Z[node][col] += alpha * sum_{t in node's projectors} C~[t] P[proj_t][col]; one warp per node.
-__global__ void __launch_bounds__(256) k_nl_add(double* __restrict__ Z, int64_t ldz, int ncol,
-                                                const int32_t* __restrict__ snode,
-                                                const int64_t* __restrict__ srow,
-                                                const int32_t* __restrict__ sproj,
-                                                const double* __restrict__ sval,
-                                                const double* __restrict__ P, int64_t nsup, double alpha) {
-  const int lane = threadIdx.x & 31;
-  const int64_t s = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int col = blockIdx.y * 32 + lane;
-  if (s >= nsup || col >= ncol) return;
-  double acc = 0.0;
-  for (int64_t t = srow[s]; t < srow[s + 1]; ++t) acc = fma(sval[t], P[(int64_t)sproj[t] * ncol + col], acc);
-  Z[(int64_t)snode[s] * ldz + col] += alpha * acc;
 }
 
 // Local part, wide form: one CTA = one cell x 32 columns (the body is shared with the batched
@@ -280,23 +224,12 @@ void local_part_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Z, int64
   else local_part_rows(h, X, ldx, Z, ldz, ncol, alpha, rows);
 }
 
-// P = h (C~^T X)
-static const double* nl_coef64(dftfe_ham h, const double* X, int64_t ldx, int ncol) {
-  double* P = (double*)ws_get(h, "nl_coef", sizeof(double) * h->nproj * (size_t)ncol);
-  double* part = (double*)ws_get(h, "nl_coef_part", sizeof(double) * h->nproj * (size_t)kNlSplits64 * ncol);
-  dim3 grid((unsigned)(h->nproj * kNlSplits64), (unsigned)((ncol + 31) / 32));
-  DFTFE_LAUNCH(k_nl_coef_part, grid, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, h->d_pval, part);
-  DFTFE_LAUNCH(k_nl_coef_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, h->stream, part, h->d_h, h->nproj, ncol, P);
-  return P;
-}
-
 // Z += alpha H~_nl X (FP64), nothing without projectors
 void nonlocal_add_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Z, int64_t ldz, int ncol, double alpha) {
   if (h->nproj <= 0) return;
-  const double* P = nl_coef64(h, X, ldx, ncol);
-  dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
-  DFTFE_LAUNCH(k_nl_add, g2, 256, 0, h->stream, Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P,
-               h->nsup, alpha);
+  double* P = (double*)ws_get(h, "nl_coef", sizeof(double) * h->nproj * (size_t)ncol);
+  nl::coef<nl::F64>(h, h->stream, X, ldx, ncol, h->d_pval, P, ncol);
+  nl::add<nl::F64>(h, h->stream, Z, ldz, ncol, h->d_sval, P, ncol, alpha);
 }
 
 void apply_combo(dftfe_ham h, const double* X, int64_t ldx, const double* Xprev, int64_t ldp,
@@ -322,12 +255,7 @@ void apply_nonlocal_fp64(dftfe_ham h, const double* X, int64_t ldx, double* Y, i
   auto* m = h->mesh;
   DFTFE_LAUNCH(k_axpby_init, nblk(m->M * ncol), 256, 0, h->stream, Y, ldy, X, ldx, nullptr, 0, m->M, ncol, 0.0,
                0.0);
-  if (h->nproj > 0) {
-    const double* P = nl_coef64(h, X, ldx, ncol);
-    dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
-    DFTFE_LAUNCH(k_nl_add, g2, 256, 0, h->stream, Y, ldy, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P,
-                 h->nsup, 1.0);
-  }
+  nonlocal_add_fp64(h, X, ldx, Y, ldy, ncol, 1.0);
 }
 
 // Eq. chebyfilter.  Unscaled: X1 = (H~ - c) X0 / e, X_{k+1} = 2 (H~ - c) X_k / e - X_{k-1}.

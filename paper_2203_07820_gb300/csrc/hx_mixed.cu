@@ -23,6 +23,7 @@
 // Every wait is bounded; on a time-out the kernel records DFTFE_ERR_TIMEOUT, drains its
 // own copies and MMAs (bounded), frees its tensor memory and returns.
 #include "internal.h"
+#include "nonlocal.cuh"
 #include "tcgen05.h"
 
 #include <cuda_bf16.h>
@@ -924,93 +925,7 @@ __global__ void k_to_f64(const float* __restrict__ Y, int64_t ldy, double* __res
   X[i * ldx + j] = (double)Y[i * ldy + j];
 }
 
-// Projector coefficients in two stages for parallelism: stage 1, CTA (a, s) sums split s
-// of projector a's support (8 warps x 4 unrolled loads per lane); stage 2 adds the splits
-// in a fixed order and scales by h_a.
-constexpr int kNlSplits = 8;
-__global__ void __launch_bounds__(256) k_nl_coef32_part(const float* __restrict__ X, int64_t ldx, int ncol,
-                                                        const int64_t* __restrict__ prow,
-                                                        const int32_t* __restrict__ pnode,
-                                                        const double* __restrict__ pval, float* __restrict__ part) {
-  // CTA (a, s): split s of projector a's support; warp w takes every 8th entry; lane l
-  // holds columns 4l..4l+3 of a 128-column tile (blockIdx.y), read as one float4
-  __shared__ float4 red[8][32];
-  const int a = blockIdx.x / kNlSplits, sidx = blockIdx.x % kNlSplits;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c0 = blockIdx.y * 128 + 4 * lane;
-  const int64_t e0 = prow[a], e1 = prow[a + 1];
-  const int64_t len = (e1 - e0 + kNlSplits - 1) / kNlSplits;
-  const int64_t s0 = e0 + sidx * len, s1 = min(e1, s0 + len);
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (c0 < ncol) {
-#pragma unroll 4
-    for (int64_t e = s0 + warp; e < s1; e += 8) {
-      const float w = (float)pval[e];
-      const float4 x = __ldg(reinterpret_cast<const float4*>(X + (int64_t)pnode[e] * ldx + c0));
-      s.x = fmaf(w, x.x, s.x); s.y = fmaf(w, x.y, s.y); s.z = fmaf(w, x.z, s.z); s.w = fmaf(w, x.w, s.w);
-    }
-  }
-  red[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0) {
-    float4 t = red[0][lane];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) {
-      const float4 u = red[w][lane];
-      t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
-    }
-    const float v[4] = {t.x, t.y, t.z, t.w};
-    for (int j = 0; j < 4; ++j)
-      if (c0 + j < ncol) part[((int64_t)blockIdx.x) * ncol + c0 + j] = v[j];
-  }
-}
-
-__global__ void k_nl_coef32_reduce(const float* __restrict__ part, const double* __restrict__ hcoup, int nproj,
-                                   int ncol, float* __restrict__ P, int ldP) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nproj * ncol) return;
-  const int a = (int)(t / ncol), col = (int)(t % ncol);
-  float s = 0.0f;
-  for (int k = 0; k < kNlSplits; ++k) s += part[((int64_t)a * kNlSplits + k) * ncol + col];
-  P[(int64_t)a * ldP + col] = (float)hcoup[a] * s;
-}
-
-// Z[node] += alpha sum_t w_t P[a_t] on the support nodes (the tensor-product form, whose cell and
-// face kernels write Z without the projectors): one warp per node, four columns per lane
-__global__ void __launch_bounds__(256) k_nl_add32(float* __restrict__ Z, int64_t ldz, int ncol,
-                                                  const int32_t* __restrict__ snode, const int64_t* __restrict__ srow,
-                                                  const int32_t* __restrict__ sproj, const double* __restrict__ sval,
-                                                  const float* __restrict__ P, int ldP, int64_t nsup, float alpha) {
-  const int64_t s = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int c = blockIdx.y * 128 + 4 * (threadIdx.x & 31);
-  if (s >= nsup || c >= ncol) return;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int64_t t = srow[s]; t < srow[s + 1]; ++t) {
-    const float w = (float)sval[t];
-    const float4 pv = *reinterpret_cast<const float4*>(P + (int64_t)sproj[t] * ldP + c);   // ldP % 4 == 0
-    acc.x = fmaf(w, pv.x, acc.x); acc.y = fmaf(w, pv.y, acc.y);
-    acc.z = fmaf(w, pv.z, acc.z); acc.w = fmaf(w, pv.w, acc.w);
-  }
-  float* z = Z + (int64_t)snode[s] * ldz + c;
-  if (c + 3 < ncol) {
-    float4 v = *reinterpret_cast<float4*>(z);
-    v.x = fmaf(alpha, acc.x, v.x); v.y = fmaf(alpha, acc.y, v.y);
-    v.z = fmaf(alpha, acc.z, v.z); v.w = fmaf(alpha, acc.w, v.w);
-    *reinterpret_cast<float4*>(z) = v;
-  } else {
-    const float a[4] = {acc.x, acc.y, acc.z, acc.w};
-    for (int j = 0; c + j < ncol; ++j) z[j] = fmaf(alpha, a[j], z[j]);
-  }
-}
-
 static unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
-
-static void nl_add32(dftfe_ham h, cudaStream_t s, float* Z, int64_t ldz, int ncol, const float* P, int ldP,
-                     float alpha) {
-  dim3 grid((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 127) / 128));
-  DFTFE_LAUNCH(k_nl_add32, grid, 256, 0, s, Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj, h->d_sval, P, ldP,
-               h->nsup, alpha);
-}
 
 // the split-precision form of this mesh: the FP32 tensor-product kernels, whose products carry
 // 24 bits where the 3-term splits carry 21, or (other quadrature rules, BF16x3) split dense products
@@ -1156,11 +1071,7 @@ static void apply_combo_mixed(dftfe_ham h, bool tf32, const uint8_t* A, int nkc,
   const int ldP = (ncol + 3) / 4 * 4;
   if (h->nproj > 0 && !kpoint) {
     P = (float*)ws_get(h, "nl_coef32", sizeof(float) * h->nproj * (size_t)ldP);
-    float* Pp = (float*)ws_get(h, "nl_coef32_part", sizeof(float) * h->nproj * (size_t)kNlSplits * ncol);
-    dim3 g1((unsigned)(h->nproj * kNlSplits), (unsigned)((ncol + 127) / 128));
-    DFTFE_LAUNCH(k_nl_coef32_part, g1, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, h->d_pval, Pp);
-    DFTFE_LAUNCH(k_nl_coef32_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, h->stream, Pp, h->d_h, h->nproj,
-                 ncol, P, ldP);
+    nl::coef<nl::F32x4>(h, h->stream, X, ldx, ncol, h->d_pval, P, ldP);
   }
   if (sf) {
     const float* v = sf_potential32(h);
@@ -1181,7 +1092,7 @@ static void apply_combo_mixed(dftfe_ham h, bool tf32, const uint8_t* A, int nkc,
       ProfScope ps(h, "cell_gemm_tf32x3");
       run();
     }
-    if (P) nl_add32(h, h->stream, Z, ldz, ncol, P, ldP, alpha);
+    if (P) nl::add<nl::F32x4>(h, h->stream, Z, ldz, ncol, h->d_sval32, P, ldP, alpha);
     if (kpoint) kpoint_add32(h, X, ldx, Z, ldz, ncol / 2, alpha, false);
     return;
   }
@@ -1537,13 +1448,7 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
       const int ncol = blk[s].ncol;
       ldP[s] = (ncol + 3) / 4 * 4;
       P[s] = (float*)ws_get(h, "nl_coef32", sizeof(float) * h->nproj * (size_t)ldP[s]);
-      float* Pp = (float*)ws_get(h, "nl_coef32_part", sizeof(float) * h->nproj * (size_t)kNlSplits * ncol);
-      const StepSys& st = steps[s][k - 1];
-      dim3 g1((unsigned)(h->nproj * kNlSplits), (unsigned)((ncol + 127) / 128));
-      DFTFE_LAUNCH(k_nl_coef32_part, g1, 256, 0, stream, sy[s].buf[st.cur], sy[s].ld32, ncol, h->d_prow, h->d_pnode,
-                   h->d_pval, Pp);
-      DFTFE_LAUNCH(k_nl_coef32_reduce, nblk((int64_t)h->nproj * ncol), 256, 0, stream, Pp, h->d_h, h->nproj, ncol,
-                   P[s], ldP[s]);
+      nl::coef<nl::F32x4>(h, stream, sy[s].buf[steps[s][k - 1].cur], sy[s].ld32, ncol, h->d_pval, P[s], ldP[s]);
     }
     for (; lsf < R.sf_launches.size() && R.sf_launches[lsf].k == k; ++lsf) {
       const auto& L = R.sf_launches[lsf];
@@ -1554,7 +1459,8 @@ static void enqueue_mixed_round(const MixedRoundPlan& R, cudaStream_t stream, in
     for (int s = 0; s < ns; ++s)
       if (sy[s].sf && P[s]) {
         const StepSys& st = steps[s][k - 1];
-        nl_add32(blk[s].h, stream, sy[s].buf[st.out], sy[s].ld32, blk[s].ncol, P[s], ldP[s], st.alpha);
+        nl::add<nl::F32x4>(blk[s].h, stream, sy[s].buf[st.out], sy[s].ld32, blk[s].ncol, blk[s].h->d_sval32, P[s],
+                           ldP[s], st.alpha);
       }
     for (int t = 0; t < ntiles; ++t) {
       for (; li < launches.size() && launches[li].k == k && launches[li].tile == t; ++li) {

@@ -128,6 +128,8 @@ struct GraphSlot {
   int64_t reinstantiations = 0;
 };
 
+constexpr int kNlGroup = 4;   // projectors summed together (one pass over their common rows)
+
 struct KernelTimer {
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;
   size_t used = 0;
@@ -169,10 +171,13 @@ struct dftfe_ham_s {
   // a3: nonlocal (CSR by projector and by node)
   int nproj = 0;
   double* d_h = nullptr;
+  int npgroup = 0;                 // runs of at most kNlGroup projectors with one node list:
+  int32_t* d_pgroup = nullptr;     // npgroup + 1 first projectors
   int64_t* d_prow = nullptr;  int32_t* d_pnode = nullptr;  double* d_pval = nullptr;
   int64_t nsup = 0;
   int32_t* d_snode = nullptr; int64_t* d_srow = nullptr;
   int32_t* d_sproj = nullptr; double* d_sval = nullptr;
+  float* d_sval32 = nullptr;       // the same in FP32
   int64_t* d_nptr_all = nullptr;   // M + 1 offsets of every node's (sproj, sval) entries
   int64_t nnz = 0;                 // projector CSR entries
   int64_t* d_sperm = nullptr;      // node-major entry t = projector-major entry d_sperm[t]

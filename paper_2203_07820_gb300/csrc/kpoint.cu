@@ -30,6 +30,7 @@
 // steps on (rho(S), Xr) give X L^-H exactly.  The Rayleigh-Ritz eigensolve is Hermitian
 // (syevd_z); its eigenvectors rotate the real views through rho(Q).
 #include "internal.h"
+#include "nonlocal.cuh"
 
 #include <cmath>
 #include <string>
@@ -97,108 +98,6 @@ __global__ void __launch_bounds__(256) k_kin_init(double2* Z, int64_t ldz,
   Z[i * ldz + c] = z;
 }
 
-// The same coefficients split over each projector's support, so that a long support does not
-// run as one latency-bound chain of dependent loads per warp: CTA (a, s) sums split s of
-// projector a's entries (warp w every 8th entry of the split, lane l complex column
-// 32 blockIdx.y + l) into part[a S + s][col]; k_nl_coefz_reduce adds the S splits in order and
-// scales by h_a.  C is float2 (the complex64 filter) or double2.
-constexpr int kNlzSplits = 8;
-template <typename C>
-__global__ void __launch_bounds__(256) k_nl_coefz_part(const C* __restrict__ X, int64_t ldx, int ncol,
-                                                       const int64_t* __restrict__ prow,
-                                                       const int32_t* __restrict__ pnode, const C* __restrict__ pval,
-                                                       C* __restrict__ part) {
-  using R = decltype(C::x);
-  __shared__ C red[8][32];
-  const int a = blockIdx.x / kNlzSplits, sidx = blockIdx.x % kNlzSplits;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int col = blockIdx.y * 32 + lane;
-  const int64_t e0 = prow[a], e1 = prow[a + 1];
-  const int64_t len = (e1 - e0 + kNlzSplits - 1) / kNlzSplits;
-  const int64_t s0 = e0 + sidx * len, s1 = min(e1, s0 + len);
-  R sr = 0, si = 0;
-  if (col < ncol) {
-#pragma unroll 4
-    for (int64_t e = s0 + warp; e < s1; e += 8) {
-      const C cv = pval[e];
-      const C xv = X[(int64_t)pnode[e] * ldx + col];
-      sr = fma(cv.x, xv.x, fma(cv.y, xv.y, sr));
-      si = fma(cv.x, xv.y, fma(-cv.y, xv.x, si));
-    }
-  }
-  C v;
-  v.x = sr;
-  v.y = si;
-  red[warp][lane] = v;
-  __syncthreads();
-  if (warp == 0 && col < ncol) {
-    R tr = 0, ti = 0;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      tr += red[w][lane].x;
-      ti += red[w][lane].y;
-    }
-    C o;
-    o.x = tr;
-    o.y = ti;
-    part[(int64_t)blockIdx.x * ncol + col] = o;
-  }
-}
-
-template <typename C>
-__global__ void k_nl_coefz_reduce(const C* __restrict__ part, const double* __restrict__ hcoup, int nproj, int ncol,
-                                  C* __restrict__ P) {
-  using R = decltype(C::x);
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nproj * ncol) return;
-  const int a = (int)(t / ncol), col = (int)(t % ncol);
-  R sr = 0, si = 0;
-  for (int k = 0; k < kNlzSplits; ++k) {
-    const C v = part[((int64_t)a * kNlzSplits + k) * ncol + col];
-    sr += v.x;
-    si += v.y;
-  }
-  const R hv = (R)hcoup[a];
-  C o;
-  o.x = hv * sr;
-  o.y = hv * si;
-  P[t] = o;
-}
-
-// P = h (C~^kH X) for ncol complex columns through the split kernels above
-template <typename C>
-static void nl_coef_z_split(dftfe_ham h, const C* X, int64_t ldx, int ncol, const C* pval, C* P) {
-  C* part = (C*)ws_get(h, sizeof(C) == 8 ? "nl_coefz32_part" : "nl_coefz_part",
-                       sizeof(C) * (size_t)h->nproj * kNlzSplits * ncol);
-  dim3 g1((unsigned)(h->nproj * kNlzSplits), (unsigned)((ncol + 31) / 32));
-  DFTFE_LAUNCH(k_nl_coefz_part<C>, g1, 256, 0, h->stream, X, ldx, ncol, h->d_prow, h->d_pnode, pval, part);
-  DFTFE_LAUNCH(k_nl_coefz_reduce<C>, nblk((int64_t)h->nproj * ncol), 256, 0, h->stream, part, h->d_h, h->nproj,
-               ncol, P);
-}
-
-// Z[node][col] += alpha sum_{t in node's projectors} C~^k_t P[proj_t][col]; one warp per node
-__global__ void __launch_bounds__(256) k_nl_add_z(double2* __restrict__ Z, int64_t ldz, int ncol,
-                                                  const int32_t* __restrict__ snode,
-                                                  const int64_t* __restrict__ srow,
-                                                  const int32_t* __restrict__ sproj,
-                                                  const double2* __restrict__ sval,
-                                                  const double2* __restrict__ P, int64_t nsup, double alpha) {
-  const int lane = threadIdx.x & 31;
-  const int64_t s = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int col = blockIdx.y * 32 + lane;
-  if (s >= nsup || col >= ncol) return;
-  double ar = 0.0, ai = 0.0;
-  for (int64_t t = srow[s]; t < srow[s + 1]; ++t) {
-    const double2 cv = sval[t];
-    const double2 pv = P[(int64_t)sproj[t] * ncol + col];
-    ar = fma(cv.x, pv.x, fma(-cv.y, pv.y, ar));
-    ai = fma(cv.x, pv.y, fma(cv.y, pv.x, ai));
-  }
-  double2* z = Z + (int64_t)snode[s] * ldz + col;
-  z->x += alpha * ar;
-  z->y += alpha * ai;
-}
-
 // FP32 forms for the mixed filter (complex64 vectors): Z += alpha (-i) sum_d G~1_d X along
 // axis d (the 1/2|k|^2 and recurrence terms are in the assembly that precedes it)
 __global__ void __launch_bounds__(256) k_kin_add32(float2* __restrict__ Z, int64_t ldz,
@@ -258,28 +157,6 @@ __global__ void __launch_bounds__(256) k_kin_add32(float2* __restrict__ Z, int64
     z->x = fmaf(alpha, si0, z->x);
     z->y = fmaf(-alpha, sr0, z->y);
   }
-}
-
-__global__ void __launch_bounds__(256) k_nl_add32_z(float2* __restrict__ Z, int64_t ldz, int ncol,
-                                                    const int32_t* __restrict__ snode,
-                                                    const int64_t* __restrict__ srow,
-                                                    const int32_t* __restrict__ sproj,
-                                                    const float2* __restrict__ sval,
-                                                    const float2* __restrict__ P, int64_t nsup, float alpha) {
-  const int lane = threadIdx.x & 31;
-  const int64_t s = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int col = blockIdx.y * 32 + lane;
-  if (s >= nsup || col >= ncol) return;
-  float ar = 0.f, ai = 0.f;
-  for (int64_t t = srow[s]; t < srow[s + 1]; ++t) {
-    const float2 cv = sval[t];
-    const float2 pv = P[(int64_t)sproj[t] * ncol + col];
-    ar = fmaf(cv.x, pv.x, fmaf(-cv.y, pv.y, ar));
-    ai = fmaf(cv.x, pv.y, fmaf(cv.y, pv.x, ai));
-  }
-  float2* z = Z + (int64_t)snode[s] * ldz + col;
-  z->x = fmaf(alpha, ar, z->x);
-  z->y = fmaf(alpha, ai, z->y);
 }
 
 __global__ void k_to_f2(float2* __restrict__ dst, const double2* __restrict__ src, int64_t n) {
@@ -410,10 +287,8 @@ void kpoint_init_terms(dftfe_ham h, const double* X, int64_t ldx, const double* 
   if (h->nproj > 0) {
     ProfScope ps(h, "nl_z");
     double2* P = (double2*)ws_get(h, "nl_coef_z", sizeof(double2) * h->nproj * (size_t)ncol);
-    nl_coef_z_split(h, (const double2*)X, ldx, ncol, (const double2*)h->d_pval_z, P);
-    dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
-    DFTFE_LAUNCH(k_nl_add_z, g2, 256, 0, h->stream, (double2*)Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj,
-                 (const double2*)h->d_sval_z, P, h->nsup, alpha);
+    nl::coef<nl::Cplx<double2>>(h, h->stream, (const double2*)X, ldx, ncol, (const double2*)h->d_pval_z, P, ncol);
+    nl::add<nl::Cplx<double2>>(h, h->stream, (double2*)Z, ldz, ncol, (const double2*)h->d_sval_z, P, ncol, alpha);
   }
 }
 
@@ -442,10 +317,8 @@ void kpoint_add32(dftfe_ham h, const float* X, int64_t ldx, float* Z, int64_t ld
   if (h->nproj > 0) {
     ProfScope ps(h, "nl_z32");
     float2* P = (float2*)ws_get(h, "nl_coef32_z", sizeof(float2) * h->nproj * (size_t)ncolz);
-    nl_coef_z_split(h, (const float2*)X, ldx / 2, ncolz, (const float2*)h->d_pval_z32, P);
-    dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncolz + 31) / 32));
-    DFTFE_LAUNCH(k_nl_add32_z, g2, 256, 0, h->stream, (float2*)Z, ldz / 2, ncolz, h->d_snode, h->d_srow, h->d_sproj,
-                 (const float2*)h->d_sval_z32, P, h->nsup, alpha);
+    nl::coef<nl::Cplx<float2>>(h, h->stream, (const float2*)X, ldx / 2, ncolz, (const float2*)h->d_pval_z32, P, ncolz);
+    nl::add<nl::Cplx<float2>>(h, h->stream, (float2*)Z, ldz / 2, ncolz, (const float2*)h->d_sval_z32, P, ncolz, alpha);
   }
 }
 
@@ -471,10 +344,8 @@ static void apply_z_df(dftfe_ham h, const double* X, int64_t ldx, double* Y, int
   if (h->nproj > 0) {
     ProfScope ps(h, "nl_z");
     double2* P = (double2*)ws_get(h, "nl_coef_z", sizeof(double2) * h->nproj * (size_t)ncol);
-    nl_coef_z_split(h, (const double2*)X, ldx, ncol, (const double2*)h->d_pval_z, P);
-    dim3 g2((unsigned)((h->nsup + 7) / 8), (unsigned)((ncol + 31) / 32));
-    DFTFE_LAUNCH(k_nl_add_z, g2, 256, 0, h->stream, (double2*)Y, ldy, ncol, h->d_snode, h->d_srow, h->d_sproj,
-                 (const double2*)h->d_sval_z, P, h->nsup, 1.0);
+    nl::coef<nl::Cplx<double2>>(h, h->stream, (const double2*)X, ldx, ncol, (const double2*)h->d_pval_z, P, ncol);
+    nl::add<nl::Cplx<double2>>(h, h->stream, (double2*)Y, ldy, ncol, (const double2*)h->d_sval_z, P, ncol, 1.0);
   }
 }
 

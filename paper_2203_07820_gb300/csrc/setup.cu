@@ -199,9 +199,11 @@ __global__ void k_scale_by_sqrt_mass(double* out, const double* chi, const int32
   if (t < n) out[t] = sqrt(mass[node[t]]) * chi[t];
 }
 
-__global__ void k_gather_vals(double* out, const double* in, const int64_t* perm, int64_t n) {
+__global__ void k_gather_vals(double* out, float* out32, const double* in, const int64_t* perm, int64_t n) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < n) out[t] = in[perm[t]];
+  if (t >= n) return;
+  out[t] = in[perm[t]];
+  out32[t] = (float)in[perm[t]];
 }
 
 static unsigned nblk(int64_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -219,7 +221,11 @@ static void free_nonlocal(dftfe_ham h) {
   cudaFree(h->d_h); cudaFree(h->d_prow); cudaFree(h->d_pnode); cudaFree(h->d_pval);
   cudaFree(h->d_snode); cudaFree(h->d_srow); cudaFree(h->d_sproj); cudaFree(h->d_sval);
   cudaFree(h->d_nptr_all); cudaFree(h->d_sperm); cudaFree(h->d_pval_z); cudaFree(h->d_sval_z);
-  cudaFree(h->d_pval_z32); cudaFree(h->d_sval_z32);
+  cudaFree(h->d_pval_z32); cudaFree(h->d_sval_z32); cudaFree(h->d_pgroup);
+  cudaFree(h->d_sval32);
+  h->d_sval32 = nullptr;
+  h->d_pgroup = nullptr;
+  h->npgroup = 0;
   h->d_pval_z32 = nullptr; h->d_sval_z32 = nullptr;
   h->d_h = nullptr; h->d_prow = nullptr; h->d_pnode = nullptr; h->d_pval = nullptr;
   h->d_snode = nullptr; h->d_srow = nullptr; h->d_sproj = nullptr; h->d_sval = nullptr;
@@ -477,6 +483,16 @@ extern "C" dftfe_status dftfe_ham_set_nonlocal(dftfe_ham h, int nproj, const dou
     sproj[t] = (int32_t)eproj[e];
   }
   srow.push_back(nnz);
+  // runs of projectors with one node list (an atom's angular channels)
+  std::vector<int32_t> group{0};
+  for (int a = 1; a < nproj; ++a) {
+    const int64_t b = rowptr[group.back()], len = rowptr[group.back() + 1] - b;
+    if (a - group.back() < kNlGroup && rowptr[a + 1] - rowptr[a] == len &&
+        std::equal(node + rowptr[a], node + rowptr[a + 1], node + b))
+      continue;
+    group.push_back(a);
+  }
+  group.push_back(nproj);
   DFTFE_CHECK_CUDA(cudaStreamSynchronize(h->stream));
   free_nonlocal(h);
   cudaStream_t s = h->stream;
@@ -484,6 +500,8 @@ extern "C" dftfe_status dftfe_ham_set_nonlocal(dftfe_ham h, int nproj, const dou
   h->nnz = nnz;
   h->nsup = (int64_t)snode.size();
   h->d_h = dev_upload(std::vector<double>(hcoup, hcoup + nproj), s);
+  h->npgroup = (int)group.size() - 1;
+  h->d_pgroup = dev_upload(group, s);
   h->d_prow = dev_upload(std::vector<int64_t>(rowptr, rowptr + nproj + 1), s);
   h->d_pnode = dev_upload(pnode, s);
   double* d_chi = dev_upload(std::vector<double>(chi, chi + nnz), s);
@@ -504,7 +522,8 @@ extern "C" dftfe_status dftfe_ham_set_nonlocal(dftfe_ham h, int nproj, const dou
   // node-major position t holds projector-major entry sperm[t] (kept for the k-point values)
   h->d_sperm = dev_upload(order, s);
   DFTFE_CHECK_CUDA(cudaMalloc(&h->d_sval, sizeof(double) * std::max<int64_t>(nnz, 1)));
-  if (nnz) DFTFE_LAUNCH(k_gather_vals, nblk(nnz), 256, 0, s, h->d_sval, h->d_pval, h->d_sperm, nnz);
+  DFTFE_CHECK_CUDA(cudaMalloc(&h->d_sval32, sizeof(float) * std::max<int64_t>(nnz, 1)));
+  if (nnz) DFTFE_LAUNCH(k_gather_vals, nblk(nnz), 256, 0, s, h->d_sval, h->d_sval32, h->d_pval, h->d_sperm, nnz);
   DFTFE_CHECK_CUDA(cudaStreamSynchronize(s));
   cudaFree(d_chi);
   ABI_END

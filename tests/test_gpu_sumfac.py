@@ -112,3 +112,69 @@ def test_batch_of_both_forms_is_bit_identical_to_single_passes(dg):
         dg.dftfe_batch_destroy(batch)
         for m in made:
             _destroy(dg, m[2], m[3])
+
+
+def _projectors(M, order, seed=3):
+    """Projectors of atoms with 1, 2, 3, 4, 5 and 9 channels on one support each: empty, one node,
+    below and above the entries a CTA stages at a time, most of the mesh.  `order` "atom" keeps an
+    atom's channels together, "channel" interleaves the atoms."""
+    rng = np.random.default_rng(seed)
+    atoms = [(1, 37), (2, 0), (3, 1), (4, 4600), (5, 530), (9, 260)]
+    rows = []
+    for a, (nch, n) in enumerate(atoms):
+        nodes = np.sort(rng.choice(M, n, replace=False))
+        rows += [(j, a, nodes, rng.standard_normal(n), 0.5 + rng.random(), rng.standard_normal((n, 3)))
+                 for j in range(nch)]
+    if order == "channel":
+        rows.sort(key=lambda r: (r[0], r[1]))
+    rowptr = np.cumsum([0] + [len(r[2]) for r in rows]).astype(np.int64)
+    return (np.array([r[4] for r in rows]), rowptr, np.concatenate([r[2] for r in rows]).astype(np.int64),
+            np.concatenate([r[3] for r in rows]), np.concatenate([r[5] for r in rows]))
+
+
+@pytest.mark.parametrize("ncol", [1, 2, 5, 16, 33, 130])
+def test_projectors_on_common_supports(dg, ncol):
+    """The nonlocal term of grouped projectors against the dense products, in both precisions, and
+    against the same projectors in an order that leaves them apart, real and complex.  Bounds: a
+    coefficient's sum has chains of at most 40 + 16 + 16 + 8 additions, a node's at most 24 terms
+    and the update, so 112 u |C| h |C|^T |X| + 2 u |Y| (u the unit roundoff of the form)."""
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 4.0), (5, 4, 4), 4)
+    try:
+        M = om.ndofs
+        X0 = synth.random_block(70 + ncol, M, ncol)
+        X = torch.from_numpy(X0).cuda()
+        Z = torch.complex(X, X.flip(0)).contiguous()
+        apply = {}
+        for prec in (dg.DFTFE_FP64, dg.DFTFE_MIXED_TF32X3):
+            apply[prec] = torch.empty_like(X)
+            dg.dftfe_ham_apply(ham, X, apply[prec], prec)
+        for order in ("atom", "channel"):
+            hc, rp, nd, chi, disp = _projectors(M, order)
+            C = np.zeros((M, len(hc)))
+            for a in range(len(hc)):
+                s = slice(rp[a], rp[a + 1])
+                C[nd[s], a] = np.sqrt(om.mass[nd[s]]) * chi[s]
+            bound = np.abs(C) @ (hc[:, None] * (np.abs(C).T @ np.abs(X0)))
+            ref = C @ (hc[:, None] * (C.T @ X0))
+            dg.dftfe_ham_set_nonlocal(ham, hc, rp, nd, chi)
+            for prec, u in ((dg.DFTFE_FP64, 2.0 ** -53), (dg.DFTFE_MIXED_TF32X3, 2.0 ** -24)):
+                Y = torch.full_like(X, float("nan"))
+                dg.dftfe_ham_apply(ham, X, Y, prec)
+                y = Y.cpu().numpy()
+                err = np.abs(y - apply[prec].cpu().numpy() - ref)
+                assert np.all(err <= 112 * u * bound + 2 * u * np.abs(y)), (order, prec)
+        dg.dftfe_ham_set_kpoint(ham, (0.2, -0.1, 0.15), disp)
+        zbound = np.abs(C) @ (hc[:, None] * (np.abs(C).T @ np.abs(Z.cpu().numpy())))
+        for prec, u in ((dg.DFTFE_FP64, 2.0 ** -53), (dg.DFTFE_MIXED_TF32X3, 2.0 ** -24)):
+            got = []
+            for order in ("atom", "channel"):
+                hc, rp, nd, chi, disp = _projectors(M, order)
+                dg.dftfe_ham_set_nonlocal(ham, hc, rp, nd, chi)
+                dg.dftfe_ham_set_kpoint(ham, (0.2, -0.1, 0.15), disp)
+                Y = torch.full_like(Z, float("nan"))
+                dg.dftfe_ham_apply_z(ham, Z, Y, prec)
+                got.append(Y.cpu().numpy())
+            # complex products: twice the terms of the real sums on each side
+            assert np.all(np.abs(got[0] - got[1]) <= 448 * u * zbound + 4 * u * np.abs(got[0])), prec
+    finally:
+        _destroy(dg, mesh, ham)
