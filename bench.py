@@ -37,14 +37,7 @@ sys.path.insert(0, ROOT)
 import synth  # noqa: E402
 
 FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12   # 152 SMs x 4 FP64 flop/clk/SM x 2.07 GHz
-# DRAM bytes (read + write) per cell per 128-column tile, from one ncu capture each on a
-# smaller workload with the same per-cell shape (profiles/cell_gemm_*_p6_block128.md); a
-# launch of this workload processes N_c / 8 cells (FP64, one colour) or all N_c cells
-# (split precision), so traffic scales with the cells.  A kernel that changed since its
-# capture has no entry here (traffic null).
-DRAM_BYTES_PER_CELL = {"cell_gemm_fp64": (124.1e6 + 10.2e6) / 64,
-                       # k_cell_tf32p<true>, one 128-column launch over 1,728 cells (p = 6)
-                       "cell_gemm_tf32x3": (1038.389e6 + 271.302e6) / 1728}
+FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12   # 152 SMs x 128 FMA/clk/SM x 2.07 GHz
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 
 
@@ -788,39 +781,43 @@ def rooflines(fam, wl, precision):
     roofs = {}
     fp64_cols = (N * wl.cheb_degree + N) if precision == "fp64" else N
     if "cell_gemm_fp64" in fam:
-        a = 2.0 * Nc * nc * nc * fp64_cols / (fam["cell_gemm_fp64"]["ms"] / 1e3) / 1e12
-        roofs["cell_gemm_fp64"] = {"kernel": "k_cell_fp64_wide (gather + FP64 cell GEMM + scatter-add)",
+        # the operator as its 1D contractions: three for the kinetic term, six for the potential
+        a = 18.0 * Nc * nc * (wl.degree + 1) * fp64_cols / (fam["cell_gemm_fp64"]["ms"] / 1e3) / 1e12
+        roofs["cell_gemm_fp64"] = {"kernel": "k_sf_cell<double> + k_sf_faces (1D contractions, FP64)",
                                    "bound": "alu", "achieved": a, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                                    "frac": a / FP64_PEAK_TFLOPS,
                                    "peak_source": "derived: 152 SMs x 4 FP64 FLOP/clk x 2.07 GHz (nominal 1.25)"}
-    for p in ("tf32x3", "bf16x3"):
-        key = "cell_gemm_" + p
-        if key not in fam:
-            continue
-        t = fam[key]["ms"] / 1e3 / fam[key]["launches"]            # one launch: one 128-column tile
+    if "cell_gemm_tf32x3" in fam:
+        t = fam["cell_gemm_tf32x3"]["ms"] / 1e3 / fam["cell_gemm_tf32x3"]["launches"]
+        byt = 3.0 * M * B * 4.0 + Nc * nc * 4.0                    # X_k, X_k-1 in, X_k+1 out; potential
+        flops = 18.0 * Nc * nc * (wl.degree + 1) * B
+        tb, ta = byt / (hbm_peak * 1e9), flops / (FP32_PEAK_TFLOPS * 1e12)
+        roofs["cell_gemm_tf32x3"] = {
+            "kernel": "k_sf_cell<float> + k_sf_faces (1D contractions, FP32, recurrence fused)",
+            "bound": "alu" if ta >= tb else "hbm",
+            "achieved": flops / t / 1e12 if ta >= tb else byt / t / 1e9,
+            "peak": FP32_PEAK_TFLOPS if ta >= tb else hbm_peak, "unit": "TFLOP/s" if ta >= tb else "GB/s",
+            "frac": max(tb, ta) / t,
+            "peak_source": "derived: 152 SMs x 128 FMA/clk x 2 x 2.07 GHz" if ta >= tb else f"{src} hbm_gbs",
+            "launch_ms": t * 1e3, "algorithmic_bytes_per_launch": byt, "algorithmic_flops_per_launch": flops,
+            "hbm_frac": tb / t, "alu_frac": ta / t, "traffic": None,
+            "units": f"one {B}-column H~X application over all {Nc} cells"}
+    if "cell_gemm_bf16x3" in fam:
+        t = fam["cell_gemm_bf16x3"]["ms"] / 1e3 / fam["cell_gemm_bf16x3"]["launches"]   # one 128-column tile
         byt = Nc * nc * nc * 4.0 + M * B * 4.0                     # FP32 H~^c stream + X once
         flops = 3 * 2.0 * Nc * nc * nc * B                         # three split products
-        tb, tt = byt / (hbm_peak * 1e9), flops / (tensor_peak[p] * 1e12)
+        tb, tt = byt / (hbm_peak * 1e9), flops / (tensor_peak["bf16x3"] * 1e12)
         tensor_bound = tt >= tb
-        kname = ("k_cell_tf32p (FP32 plane split on chip, A from TMEM" if p == "tf32x3"
-                 else "k_cell_mixed<bf16x3> (pre-split tiles") + ", tcgen05, FP32 TMEM accumulation)"
-        r = {"kernel": kname,
-             "bound": "tensor" if tensor_bound else "hbm",
-             "achieved": flops / t / 1e12 if tensor_bound else byt / t / 1e9,
-             "peak": tensor_peak[p] if tensor_bound else hbm_peak,
-             "unit": "TFLOP/s" if tensor_bound else "GB/s",
-             "frac": max(tb, tt) / t,
-             "peak_source": (f"{src} bf16 sustained" + (" x nominal tf32/bf16 (1.1/2.25)" if p == "tf32x3" else ""))
-                            if tensor_bound else f"{src} hbm_gbs",
-             "launch_ms": t * 1e3,
-             "algorithmic_bytes_per_launch": byt, "algorithmic_flops_per_launch": flops,
-             "hbm_achieved_gbs": byt / t / 1e9, "hbm_frac": tb / t,
-             "tensor_achieved_tflops": flops / t / 1e12, "tensor_frac": tt / t,
-             "units": f"one launch = one {B}-column H~X application over all {Nc} cells"}
-        per_cell = DRAM_BYTES_PER_CELL.get(key) if wl.degree == 6 else None
-        r["traffic"] = per_cell * Nc if per_cell else None
-        r["traffic_over_algorithmic"] = r["traffic"] / byt if per_cell else None
-        roofs[key] = r
+        roofs["cell_gemm_bf16x3"] = {
+            "kernel": "k_cell_mixed<bf16x3> (pre-split tiles, tcgen05, FP32 TMEM accumulation)",
+            "bound": "tensor" if tensor_bound else "hbm",
+            "achieved": flops / t / 1e12 if tensor_bound else byt / t / 1e9,
+            "peak": tensor_peak["bf16x3"] if tensor_bound else hbm_peak,
+            "unit": "TFLOP/s" if tensor_bound else "GB/s", "frac": max(tb, tt) / t,
+            "peak_source": f"{src} bf16 sustained" if tensor_bound else f"{src} hbm_gbs",
+            "launch_ms": t * 1e3, "algorithmic_bytes_per_launch": byt, "algorithmic_flops_per_launch": flops,
+            "hbm_frac": tb / t, "tensor_frac": tt / t, "traffic": None,
+            "units": f"one launch = one {B}-column H~X application over all {Nc} cells"}
     if "assemble32" in fam:
         t = fam["assemble32"]["ms"] / 1e3 / fam["assemble32"]["launches"]
         byt = Nc * nc * B * 4.0 + 3.0 * M * B * 4.0      # per-cell products in; X_k, X_k-1 in; Z out
@@ -828,12 +825,12 @@ def rooflines(fam, wl, precision):
                                "bound": "hbm", "achieved": byt / t / 1e9, "peak": hbm_peak, "unit": "GB/s",
                                "frac": byt / t / 1e9 / hbm_peak, "peak_source": f"{src} hbm_gbs"}
     if "cell_gemm_df" in fam:
-        a = 2.0 * Nc * nc * nc * N / (fam["cell_gemm_df"]["ms"] / 1e3) / 1e12
-        fp32_peak = 152 * 128 * 2 * 2.07e9 / 1e12
-        roofs["cell_gemm_df"] = {"kernel": "k_cell_df_tiled (float-pair FP64-accurate cell products, W = H~X)",
-                                 "bound": "alu", "achieved": a, "peak": fp32_peak / 12.0, "unit": "TFLOP/s",
-                                 "frac": a / (fp32_peak / 12.0),
-                                 "peak_source": "derived: FP32 peak 152 SMs x 128 FMA/clk x 2 x 2.07 GHz / 12 "
+        a = 18.0 * Nc * nc * (wl.degree + 1) * N / (fam["cell_gemm_df"]["ms"] / 1e3) / 1e12
+        # a float-pair multiply-add: 4 FP32 operations for the product, 9 for the sum
+        roofs["cell_gemm_df"] = {"kernel": "k_sf_cell float pairs + k_sf_faces (FP64-accurate 1D contractions, W = H~X)",
+                                 "bound": "alu", "achieved": a, "peak": FP32_PEAK_TFLOPS / 13.0, "unit": "TFLOP/s",
+                                 "frac": a / (FP32_PEAK_TFLOPS / 13.0),
+                                 "peak_source": "derived: FP32 peak 152 SMs x 128 FMA/clk x 2 x 2.07 GHz / 13 "
                                                 "FP32 instructions per float-pair multiply-add"}
     if "cell_gemm_slices" in fam:
         # W = H~X from exact digit products: 21 bf16 digit products per multiply-add; the

@@ -57,13 +57,17 @@ typedef enum {
   DFTFE_MIXED_BF16X3 = 1,  /* filter: cell products as 3-term BF16 splits (hi*hi + hi*lo +
                               lo*hi) on the tensor cores (tcgen05), FP32 accumulation, FP32
                               vectors; CholGS, Rayleigh-Ritz and residuals in FP64 */
-  DFTFE_MIXED_TF32X3 = 2,  /* as above with 3-term TF32 splits (about 2^-21 relative per
-                              product instead of 2^-16) */
-  DFTFE_FP64_FLOAT_PAIRS = 3, /* dftfe_ham_apply(_z) only: FP64-accurate cell products from
+  DFTFE_MIXED_TF32X3 = 2,  /* filter: the operator as FP32 1D contractions (24-bit products),
+                              FP32 vectors; with another quadrature rule than the default or
+                              the nodal one, cell products as 3-term TF32 splits (about 2^-21
+                              relative per product).  CholGS and Rayleigh-Ritz as below */
+  DFTFE_FP64_FLOAT_PAIRS = 3, /* dftfe_ham_apply(_z) only: FP64-accurate local operator from
                               pairs of floats (error-free products, TwoSum accumulation, about
                               44 significant bits) on the FP32 pipes; FP64 in and out */
-  DFTFE_FP64_SLICES = 4     /* dftfe_ham_apply(_z) only: FP64-accurate cell products on the
-                              tensor cores from exact digit products: each cell-matrix row and
+  DFTFE_FP64_SLICES = 4     /* dftfe_ham_apply(_z) only: FP64-accurate local operator; default
+                              and nodal rules: float-pair 1D contractions of columns scaled by
+                              their largest entry's exponent; other rules: cell products on
+                              the tensor cores from exact digit products: each cell-matrix row and
                               each column of X as 41-bit fixed point (relative to its largest
                               entry) in six 7-bit bf16 digits, the 21 digit products of order
                               <= 5 accumulated exactly in FP32 (each sum stays below 2^24),
@@ -72,7 +76,7 @@ typedef enum {
   /* In dftfe_cholgs, dftfe_rayleigh_ritz and the pass, either mixed value selects the
      mixed overlap / projection / rotation of Sec. 3.2: diagonal entries of S and H^ and
      the diagonal part of each rotation in FP64, off-diagonal parts in FP32; W = H~X
-     for the projection and the residuals uses the exact digit products of
+     for the projection and the residuals takes the form of
      DFTFE_FP64_SLICES (the float pairs of DFTFE_FP64_FLOAT_PAIRS beyond degree 7; split
      products there would move the Ritz values by 1e-6 to 2e-6 Ha); the Cholesky
      factorisation and the eigensolve stay FP64. */
@@ -125,16 +129,16 @@ dftfe_status dftfe_mesh_destroy(dftfe_mesh mesh);
 /* ---------------------------------------------------------------- Hamiltonian */
 
 /* Build the device operator state on the current CUDA device: cell -> global
- * map, lumped mass M (a1), the shared GLL stiffness, the packed product table
- * P of Eq. gemmLoc, and storage for the N_c dense cell matrices.  stream: a
+ * map, lumped mass M (a1), the shared GLL stiffness, and storage for the N_c dense
+ * cell matrices.  stream: a
  * cudaStream_t (NULL = legacy default stream) on which every later call of this
  * ham runs.  The mesh must outlive the ham. */
 dftfe_status dftfe_ham_create(dftfe_mesh mesh, void* stream, dftfe_ham* out);
 
 /* A second ham over src's mesh, on src's stream, that uses src's local operator: the cell
  * matrices H~^c that dftfe_ham_set_potential(src, ...) forms and every form the library
- * derives from them (the FP32 plane of the split products, the digit rows of the exact-slice
- * products, the float pairs), built once on first use and read by both.  The local term
+ * derives from them (the scaled potential in FP64, FP32 and float pairs; the FP32 plane of the
+ * split products, the digit rows of the exact-slice products), built once on first use and read by both.  The local term
  * -1/2 lap + V_loc is the same at every Bloch k-point of a system (Sec. 2.1: only the k terms
  * and the projector phases depend on k), so the k-point hams of one system made this way
  * hold one copy of it instead of one each.  The new ham has its own nonlocal term, k-point,
@@ -169,16 +173,18 @@ dftfe_status dftfe_ham_destroy(dftfe_ham ham);
 dftfe_status dftfe_ham_export(dftfe_ham ham, double* mass, int32_t* cell_map,
                               int64_t c0, int64_t count, double* cell_mats);
 
-/* Y = H~ X for an M x ncol block (a4 + a5; Eq. celldgemm and Alg. 4): gather to
- * cells, dense per-cell product, colour-ordered scatter-add, plus C~ h C~^T X.
+/* Y = H~ X for an M x ncol block (a4 + a5; Alg. 4): per cell the three kinetic and six
+ * potential 1D contractions, sums over shared faces in a fixed order, plus C~ h C~^T X (quadrature
+ * rules other than the default and the nodal one: Eq. celldgemm's dense per-cell products).
  * X and Y in DEVICE memory, must not overlap.  prec selects the FP64 cell kernel, the
- * split-precision tensor-core kernel (FP32 inside, converted at both ends; at most 512
+ * split-precision kernel (FP32 inside, converted at both ends; at most 512
  * nodes per cell, i.e. p <= 7), or one of the two FP64-accurate forms used for W in the
  * mixed passes (DFTFE_FP64_FLOAT_PAIRS; DFTFE_FP64_SLICES, p <= 7). */
 dftfe_status dftfe_ham_apply(dftfe_ham ham, const double* X, int64_t ldx,
                              double* Y, int64_t ldy, int ncol, dftfe_precision prec);
 
-/* Autotuner (no counterpart in the paper).  With enable = 1, the first FP64 cell-product
+/* Autotuner (no counterpart in the paper).  The 1D-contraction kernels have one launch shape, which
+ * the queries report with its time.  For the dense cell products, with enable = 1, the first FP64 cell-product
  * pass over the mesh for each column count (real columns: 2 ncol for the _z calls) times
  * every launch shape of the FP64 cell kernel -- 64, 128, ... rows of a cell per CTA, and the
  * built-in heuristic -- on the caller's block into a scratch output and keeps the fastest
@@ -368,8 +374,8 @@ dftfe_status dftfe_ham_set_kpoint(dftfe_ham ham, const double* k, const double* 
 dftfe_status dftfe_mesh_kpoint_stencil(dftfe_mesh mesh, const double* k, double* table);
 
 /* Y = H~^k X for complex M x ncol blocks (X, Y DEVICE, not overlapping).  prec as in
- * dftfe_ham_apply: FP64; DFTFE_FP64_SLICES or DFTFE_FP64_FLOAT_PAIRS (local part from
- * exact digit products or float pairs on the real view, k terms and projectors FP64: the
+ * dftfe_ham_apply: FP64; DFTFE_FP64_SLICES or DFTFE_FP64_FLOAT_PAIRS (local part in
+ * the form of that precision on the real view, k terms and projectors FP64: the
  * W of a mixed complex pass uses the former); or a split precision (FP32 complex inside:
  * the split cell products act on the real view, the k terms and projectors in FP32). */
 dftfe_status dftfe_ham_apply_z(dftfe_ham ham, const double* X, int64_t ldx, double* Y,
@@ -456,9 +462,8 @@ dftfe_status dftfe_batch_create(const dftfe_ham* hams, int nsys, dftfe_batch* ou
  * Rayleigh-Ritz, residuals) run one after another and share one workspace that the batch owns
  * (sized by the largest system, freed by dftfe_batch_destroy), so a batch of many k-point
  * items holds one set of tail buffers instead of one per item.  prec is DFTFE_FP64 (shared FP64
- * launches as above) or DFTFE_MIXED_TF32X3: the split-precision filter of Sec. 4.3's cell
- * products on the tensor cores, where per Chebyshev step ONE persistent cell-product launch
- * per FE degree covers every cell of every system still filtering (a work list of
+ * launches as above) or DFTFE_MIXED_TF32X3: the split-precision filter,
+ * where per Chebyshev step one cell launch per FE degree covers every cell of every system still filtering (a work list of
  * (system, cell) pairs; complex items as complex64 through their real view), the assembly
  * with the recurrence, the nonlocal and k-point terms run per system, and CholGS /
  * Rayleigh-Ritz as dftfe_chfsi_pass in that precision.  Either way the results are

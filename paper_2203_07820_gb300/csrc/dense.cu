@@ -700,6 +700,7 @@ __host__ __device__ constexpr int lz_segments(int nv) { return nv >= 5 ? 1 : nv 
 __global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* __restrict__ Vm, int nv,
                                                                 const double* __restrict__ w, int64_t M,
                                                                 double* __restrict__ part) {
+  after_previous();
   const int segs = lz_segments(nv), lane = threadIdx.x & 31;
   const int64_t rows = (M + gridDim.x - 1) / gridDim.x;
   const int64_t i0 = blockIdx.x * rows, i1 = min(M, i0 + rows), len = (rows + segs - 1) / segs;
@@ -716,9 +717,11 @@ __global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* __
   }
 }
 
+// (A last-CTA-adds form of the pair measured 11.2 us against 4.3 + 3.4 at 64,000 entries.)
 // out[v] = sum of part's n entries of vector v = blockIdx.x (fixed order); mode 1 stores sqrt.
 __global__ void __launch_bounds__(128) k_multidot_final(const double* __restrict__ part, int n, double* out, int mode) {
   __shared__ double red[5];
+  after_previous();
   double s = 0.0;
   for (int b = threadIdx.x; b < n; b += 128) s += part[(int64_t)blockIdx.x * n + b];
   s = block_sum<128>(s, red);
@@ -726,13 +729,14 @@ __global__ void __launch_bounds__(128) k_multidot_final(const double* __restrict
 }
 static void multidot(cudaStream_t s, const double* Vm, int nv, const double* w, int64_t M, double* part, double* out,
                      int mode) {
-  DFTFE_LAUNCH(k_multidot_partial, LZ_G, 32 * LZ_W, 0, s, Vm, nv, w, M, part);
-  DFTFE_LAUNCH(k_multidot_final, (unsigned)nv, 128, 0, s, part, LZ_G * lz_segments(nv), out, mode);
+  launch_after(k_multidot_partial, LZ_G, 32 * LZ_W, 0, s, Vm, nv, w, M, part);
+  launch_after(k_multidot_final, (unsigned)nv, 128, 0, s, part, LZ_G * lz_segments(nv), out, mode);
 }
 
 // w = (w - a v) - b u   (a = *pa, b = *pb or 0)
 __global__ void k_lz_three_term(double* w, const double* v, const double* u, const double* pa,
                                 const double* pb, int64_t M) {
+  after_previous();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= M) return;
   double x = w[i] - pa[0] * v[i];
@@ -742,6 +746,7 @@ __global__ void k_lz_three_term(double* w, const double* v, const double* u, con
 
 // w -= sum_v hcoef[v] V[v]
 __global__ void k_lz_reorth(double* w, const double* Vm, int nv, const double* hcoef, int64_t M) {
+  after_previous();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= M) return;
   double s = 0.0;
@@ -751,6 +756,7 @@ __global__ void k_lz_reorth(double* w, const double* Vm, int nv, const double* h
 
 // out = w / *pn (0 if the norm is 0)
 __global__ void k_lz_scale(double* out, const double* w, const double* pn, int64_t M) {
+  after_previous();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= M) return;
   const double n = pn[0];
@@ -837,20 +843,20 @@ void lanczos(dftfe_ham h, int k, const double* v0, uint64_t seed, double* out3, 
   if (v0) DFTFE_CHECK_CUDA(cudaMemcpyAsync(w, v0, sizeof(double) * M, cudaMemcpyDeviceToDevice, s));
   else random_uniform(s, w, M, seed, 0);
   multidot(s, w, 1, w, M, part, nrm, 1);
-  DFTFE_LAUNCH(k_lz_scale, nblk(M), 256, 0, s, Vm, w, nrm, M);
+  launch_after(k_lz_scale, nblk(M), 256, 0, s, Vm, w, nrm, M);
   for (int j = 0; j < k; ++j) {
     double* vj = Vm + (int64_t)j * M;
     if (cplx) apply_combo_z(h, vj, 1, nullptr, 0, w, 1, 1, 1.0, 0.0, 0.0);
     else apply_combo(h, vj, 1, nullptr, 0, w, 1, 1, 1.0, 0.0, 0.0);
     multidot(s, vj, 1, w, M, part, alpha + j, 0);
-    DFTFE_LAUNCH(k_lz_three_term, nblk(M), 256, 0, s, w, vj, j > 0 ? vj - M : nullptr, alpha + j,
+    launch_after(k_lz_three_term, nblk(M), 256, 0, s, w, vj, j > 0 ? vj - M : nullptr, alpha + j,
                  j > 0 ? beta + j - 1 : alpha + j, M);
     for (int rep = 0; rep < 2; ++rep) {
       multidot(s, Vm, j + 1, w, M, part, hco, 0);
-      DFTFE_LAUNCH(k_lz_reorth, nblk(M), 256, 0, s, w, Vm, j + 1, hco, M);
+      launch_after(k_lz_reorth, nblk(M), 256, 0, s, w, Vm, j + 1, hco, M);
     }
     multidot(s, w, 1, w, M, part, beta + j, 1);
-    DFTFE_LAUNCH(k_lz_scale, nblk(M), 256, 0, s, Vm + (int64_t)(j + 1) * M, w, beta + j, M);
+    launch_after(k_lz_scale, nblk(M), 256, 0, s, Vm + (int64_t)(j + 1) * M, w, beta + j, M);
   }
   DFTFE_LAUNCH(k_lz_bound, 1, 64, 0, s, alpha, beta, k, d_out, st);
   int hst = 0;

@@ -121,10 +121,13 @@ __global__ void __cluster_dims__(kSplits, 1, 1) __launch_bounds__(32 * kWarps)
               const typename T::W* __restrict__ pval, const double* __restrict__ hcoup,
               typename T::E* __restrict__ P, int64_t ldP) {
   using V = typename T::V;
-  __shared__ V red[kWarps][LC];
-  __shared__ typename T::S val[kNlGroup][kChunk];
-  __shared__ int32_t node[kChunk];
+  constexpr size_t kRed = sizeof(V) * kNlGroup * kWarps * LC, kVal = sizeof(typename T::S) * kNlGroup * kChunk;
+  __shared__ alignas(16) uint8_t buf[kRed > kVal ? kRed : kVal];
+  auto val = reinterpret_cast<typename T::S(*)[kChunk]>(buf);       // while the rows are summed
+  auto red = reinterpret_cast<V(*)[kWarps][LC]>(buf);               // then the warps' sums
   __shared__ V part[kNlGroup][LC];
+  __shared__ int32_t node[kChunk];
+  after_previous();
   auto cluster = cooperative_groups::this_cluster();
   const int g = blockIdx.x / kSplits, sidx = blockIdx.x % kSplits;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lc = lane % LC;
@@ -157,26 +160,16 @@ __global__ void __cluster_dims__(kSplits, 1, 1) __launch_bounds__(32 * kWarps)
 #pragma unroll
       for (int j = 0; j < kNlGroup; ++j) T::add(acc[j], T::shfl(acc[j], o));
   }
-  // the warps' sums of one projector after the other, in the same order whatever the group
+  __syncthreads();
+  if (lane < LC)
 #pragma unroll
-  for (int j = 0; j < kNlGroup; ++j) {
-    if (j >= cnt) break;
-    if (j) __syncthreads();
-    if (lane < LC) red[warp][lane] = acc[j];
-    __syncthreads();
-    if (warp < 8 && lane < LC) {
-      V t = red[warp][lane];
+    for (int j = 0; j < kNlGroup; ++j) red[j][warp][lane] = acc[j];
+  __syncthreads();
+  if (warp < cnt && lane < LC) {
+    V t = red[warp][0][lane];
 #pragma unroll
-      for (int w = 8; w < kWarps; w += 8) T::add(t, red[warp + w][lane]);
-      red[warp][lane] = t;
-    }
-    __syncthreads();
-    if (warp == 0 && lane < LC) {
-      V t = red[0][lane];
-#pragma unroll
-      for (int w = 1; w < 8; ++w) T::add(t, red[w][lane]);
-      part[j][lane] = t;
-    }
+    for (int w = 1; w < kWarps; ++w) T::add(t, red[warp][w][lane]);
+    part[warp][lane] = t;
   }
   cluster.sync();
   if (sidx == 0 && warp < cnt && lane < LC && in) {
@@ -197,6 +190,7 @@ __global__ void __launch_bounds__(256) k_nl_add(typename T::E* __restrict__ Z, i
                                                 const typename T::S* __restrict__ sval,
                                                 const typename T::E* __restrict__ P, int64_t ldP, int64_t nsup,
                                                 double alpha) {
+  after_previous();
   const int64_t s = blockIdx.x * (int64_t)(256 / LC) + threadIdx.x / LC;
   const int c = (blockIdx.y * LC + threadIdx.x % LC) * T::kCols;
   if (s >= nsup || c >= ncol) return;
@@ -219,13 +213,13 @@ void coef(dftfe_ham h, cudaStream_t stream, const typename T::E* X, int64_t ldx,
   const unsigned gx = (unsigned)(h->npgroup * kSplits);
   if constexpr (T::kCols == 1) {
     if (ncol == 1) {
-      DFTFE_LAUNCH((k_nl_coef<T, 1>), dim3(gx), 32 * kWarps, 0, stream, X, ldx, ncol, h->d_pgroup, h->d_prow,
+      launch_after(k_nl_coef<T, 1>, dim3(gx), 32 * kWarps, 0, stream, X, ldx, ncol, h->d_pgroup, h->d_prow,
                    h->d_pnode, pval, h->d_h, P, ldP);
       return;
     }
   }
   constexpr int kTile = T::kLanes * T::kCols;
-  DFTFE_LAUNCH((k_nl_coef<T, T::kLanes>), dim3(gx, (unsigned)((ncol + kTile - 1) / kTile)), 32 * kWarps, 0, stream, X, ldx,
+  launch_after(k_nl_coef<T, T::kLanes>, dim3(gx, (unsigned)((ncol + kTile - 1) / kTile)), 32 * kWarps, 0, stream, X, ldx,
                ncol, h->d_pgroup, h->d_prow, h->d_pnode, pval, h->d_h, P, ldP);
 }
 
@@ -234,13 +228,13 @@ void add(dftfe_ham h, cudaStream_t stream, typename T::E* Z, int64_t ldz, int nc
          const typename T::E* P, int64_t ldP, double alpha) {
   if constexpr (T::kCols == 1) {
     if (ncol == 1) {
-      DFTFE_LAUNCH((k_nl_add<T, 1>), (unsigned)((h->nsup + 255) / 256), 256, 0, stream, Z, ldz, ncol, h->d_snode,
+      launch_after(k_nl_add<T, 1>, (unsigned)((h->nsup + 255) / 256), 256, 0, stream, Z, ldz, ncol, h->d_snode,
                    h->d_srow, h->d_sproj, sval, P, ldP, h->nsup, alpha);
       return;
     }
   }
   constexpr int kTile = T::kLanes * T::kCols, kNodes = 256 / T::kLanes;
-  DFTFE_LAUNCH((k_nl_add<T, T::kLanes>),
+  launch_after(k_nl_add<T, T::kLanes>,
                dim3((unsigned)((h->nsup + kNodes - 1) / kNodes), (unsigned)((ncol + kTile - 1) / kTile)), 256, 0,
                stream, Z, ldz, ncol, h->d_snode, h->d_srow, h->d_sproj, sval, P, ldP, h->nsup, alpha);
 }

@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(SfCfg<W, N>::THREADS, SfCfg<W, N>::MINB)
     return wl;
   };
   int cur = 0;
+  after_previous();
   int wloc = load(0, (int)blockIdx.x);
   __syncthreads();
   Place q = place(its[0], first[0], wloc);
@@ -422,17 +423,20 @@ __global__ void __launch_bounds__(SfCfg<W, N>::THREADS, SfCfg<W, N>::MINB)
 
 // Nodes on cell surfaces: Z = s1 X + s2 Xp + alpha (sum of the face-buffer entries of the 2, 4 or 8
 // cells that hold the node, z lowest first inside y inside x).  One CTA per cell takes the
-// surface nodes it owns, VEC columns per thread; bound by memory.
+// surface nodes it owns, VEC columns per thread; bound by memory: 200 us for the 1.03 GB of 16^3 cells x
+// 128 FP32 columns at p = 6 (76 % of the copy bandwidth).  Five CTAs per SM: at four (52 to 56
+// registers) 229 us.
 template <typename T, int VEC> struct alignas(sizeof(T) * VEC) SfVec {
   T v[VEC];
 };
 template <typename T, int N, int VEC>
-__global__ void __launch_bounds__(256) k_sf_faces(const __grid_constant__ sf::Item<T> one,
-                                                  const sf::Item<T>* __restrict__ items,
-                                                  const int2* __restrict__ work) {
+__global__ void __launch_bounds__(256, 5) k_sf_faces(const __grid_constant__ sf::Item<T> one,
+                                                     const sf::Item<T>* __restrict__ items,
+                                                     const int2* __restrict__ work) {
   using V = SfVec<T, VEC>;
   constexpr int p = N - 1, NS = sf::surface_count<N>(), NO = sf::owned_count<N>();
   __shared__ sf::Item<T> it;
+  after_previous();
   const int cell = load_item(it, one, items, work, (int)blockIdx.x);
   __syncthreads();
   const int cyz = cell / it.nx, cx = cell - cyz * it.nx, cz = cyz / it.ny, cy = cyz - cz * it.ny;
@@ -820,7 +824,7 @@ static void launch_cell(cudaStream_t s, int sm, const sf::Tables<typename SfVec_
   // flight; FP64: one CTA per item, since the FP64 pipe hides the loads and a fixed deal of long
   // items would leave it idle at the end
   const unsigned grid = (unsigned)(W <= 1 ? n : std::min<int64_t>(n, (int64_t)sm * Cfg::MINB));
-  DFTFE_LAUNCH((k_sf_cell<T, W, N, NODAL, KPT>), grid, Cfg::THREADS, Cfg::smem(NODAL), s, tab, G, one, items, work,
+  launch_after(k_sf_cell<T, W, N, NODAL, KPT>, grid, Cfg::THREADS, Cfg::smem(NODAL), s, tab, G, one, items, work,
                (int)n);
 }
 
@@ -845,7 +849,7 @@ void sf_launch64(cudaStream_t s, int sm, const dftfe_mesh_s* m, const sf::Item<d
     const auto& t = mesh_tables<double, N>(m);
     if (m->vquad == 1) launch_cell<double, 1, N, true, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
     else launch_cell<double, 1, N, false, false>(s, sm, t.tab, t.G, one, items, cell_work, ncell_work);
-    DFTFE_LAUNCH((k_sf_faces<double, N, 1>), (unsigned)nface_work, 256, 0, s, one, items, face_work);
+    launch_after(k_sf_faces<double, N, 1>, (unsigned)nface_work, 256, 0, s, one, items, face_work);
   });
 }
 
@@ -873,7 +877,7 @@ void sf_launch32(cudaStream_t s, int sm, const dftfe_mesh_s* m, bool kpoint, int
       } else {
         cell(std::integral_constant<int, 2>());
       }
-      DFTFE_LAUNCH((k_sf_faces<float, N, 4>), (unsigned)nface_work, 256, 0, s, one, items, face_work);
+      launch_after(k_sf_faces<float, N, 4>, (unsigned)nface_work, 256, 0, s, one, items, face_work);
     }
   });
 }
@@ -919,7 +923,7 @@ void sf_local_pairs(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_
         launch_cell<double, 0, N, true, false>(h->stream, h->sm_count, t.tab, t.G, one, nullptr, nullptr, n);
       else
         launch_cell<double, 0, N, false, false>(h->stream, h->sm_count, t.tab, t.G, one, nullptr, nullptr, n);
-      DFTFE_LAUNCH((k_sf_faces<double, N, 1>), (unsigned)m->Nc, 256, 0, h->stream, one, nullptr, nullptr);
+      launch_after(k_sf_faces<double, N, 1>, (unsigned)m->Nc, 256, 0, h->stream, one, nullptr, nullptr);
     });
   }
 }
