@@ -58,20 +58,33 @@ __device__ __forceinline__ void slices3(float f, uint32_t& s1, uint32_t& s2, uin
   s3 = tc::tf32_rn_bits(__float_as_uint(r1 - __uint_as_float(s2)));
 }
 
-// the six slice products of one 32-deep chunk into accumulator d (fresh), the smallest first: an
-// MMA truncates at the accumulator's size, which stays 2^-11 of the result's until the last four
-__device__ __forceinline__ void chunk_mma(uint32_t d, uint32_t a0, uint32_t b0) {
+// The six slice products of one 32-deep chunk into accumulator d (fresh).  An MMA truncates at the
+// accumulator's size, a bias that the overlap and the rotation by L^-T carry into X^T X - 1; there
+// the smallest products go first, and only the last four of 24 MMAs truncate at the result's size
+// (1.7e-6 to 5.6e-7 for a filtered 14k x 72 block, same time).  The projection and the rotation by
+// Q keep the k-step order: an orthonormal block's Ritz vectors within a near-degenerate cluster are
+// fixed by that rounding alone, and stay those of earlier releases.
+__device__ __forceinline__ void chunk_mma(uint32_t d, uint32_t a0, uint32_t b0, bool small_first) {
   const uint32_t id = tc::idesc(2u, 128, 128);
+  auto product = [&](int ks, int sa, int sb, bool more) {
+    const uint32_t o = ks * 32;
+    tc::mma_tf32(d, tc::sdesc(a0 + sa * kTile + o), tc::sdesc(b0 + sb * kTile + o), id, more ? 1u : 0u);
+  };
+  if (small_first) {
 #pragma unroll
-  for (int order = 2; order >= 0; --order)
+    for (int order = 2; order >= 0; --order)
 #pragma unroll
-    for (int ks = 0; ks < 4; ++ks) {
-      const uint32_t o = ks * 32;
+      for (int ks = 0; ks < 4; ++ks)
 #pragma unroll
-      for (int sa = 0; sa <= order; ++sa)
-        tc::mma_tf32(d, tc::sdesc(a0 + sa * kTile + o), tc::sdesc(b0 + (order - sa) * kTile + o), id,
-                     order < 2 || ks > 0 || sa > 0 ? 1u : 0u);
-    }
+        for (int sa = 0; sa <= order; ++sa) product(ks, sa, order - sa, order < 2 || ks > 0 || sa > 0);
+  } else {
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+      for (int order = 0; order <= 2; ++order)
+#pragma unroll
+        for (int sa = 0; sa <= order; ++sa) product(ks, sa, order - sa, ks > 0 || order > 0);
+  }
 }
 
 // epilogue: add chunk kc's 32 x 128 accumulator block of this warp's quadrant into acc
@@ -189,7 +202,7 @@ __global__ void __launch_bounds__(st::kThreads, 1) k_rot_tc(const double* __rest
         if (!mbar_wait(&sh->b_full[s], (kc / kStages) & 1, abort, err)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a0 = smem_u32(base + s * kStage);
-        chunk_mma(tmem + (uint32_t)(128 * buf), a0, a0 + kOperand);
+        chunk_mma(tmem + (uint32_t)(128 * buf), a0, a0 + kOperand, upper != 0);
         tc_commit(&sh->empty[s]);
         tc_commit(&sh->acc_full[buf]);
       }
@@ -345,7 +358,7 @@ __global__ void __launch_bounds__(st::kThreads, 1) k_gram_tc(const double* __res
         if (!mbar_wait(&sh->a_full[s], (kc / kStages) & 1, abort, err)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a0 = smem_u32(base + s * kStage);
-        chunk_mma(tmem + (uint32_t)(128 * buf), a0, a0 + kOperand);
+        chunk_mma(tmem + (uint32_t)(128 * buf), a0, a0 + kOperand, A == B);
         tc_commit(&sh->empty[s]);
         tc_commit(&sh->acc_full[buf]);
       }
