@@ -697,9 +697,8 @@ constexpr int LZ_W = 8;            // warps of each
 __host__ __device__ constexpr int lz_segments(int nv) { return nv >= 5 ? 1 : nv >= 3 ? 2 : nv == 2 ? 4 : 8; }
 // part[(v*G + b)*segs + q] = partial dot of V[v] (stride M) with w over segment q of block b's rows: one
 // warp per (vector, segment), so that neither one vector nor twenty leave warps idle.
-__global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* __restrict__ Vm, int nv,
-                                                                const double* __restrict__ w, int64_t M,
-                                                                double* __restrict__ part) {
+__global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* Vm, int nv, const double* w, int64_t M,
+                                                                double* part) {
   after_previous();
   const int segs = lz_segments(nv), lane = threadIdx.x & 31;
   const int64_t rows = (M + gridDim.x - 1) / gridDim.x;
@@ -719,7 +718,7 @@ __global__ void __launch_bounds__(32 * LZ_W) k_multidot_partial(const double* __
 
 // (A last-CTA-adds form of the pair measured 11.2 us against 4.3 + 3.4 at 64,000 entries.)
 // out[v] = sum of part's n entries of vector v = blockIdx.x (fixed order); mode 1 stores sqrt.
-__global__ void __launch_bounds__(128) k_multidot_final(const double* __restrict__ part, int n, double* out, int mode) {
+__global__ void __launch_bounds__(128) k_multidot_final(const double* part, int n, double* out, int mode) {
   __shared__ double red[5];
   after_previous();
   double s = 0.0;

@@ -56,7 +56,11 @@ extern std::atomic<int64_t> g_launches;
 // writes are visible.  For the chains of short dependent kernels (a filter step, a Lanczos step),
 // where the gap between two launches is of the size of the kernels: FP32 filter of 32 columns,
 // 14k DoFs, 40 launches: 400 us without it, 277 with; Lanczos bound at 64,000 DoFs, 323 launches:
-// 2,540 and 1,820.  A stream under capture gets an ordinary launch, and so an ordinary graph edge.
+// 2,540 and 1,820.  What an earlier kernel of the stream writes is read by plain loads, through
+// parameters without __restrict__: __ldg and const __restrict__ loads take the read-only path, which is
+// defined only for memory that nobody writes while the kernel lives, and loads through either may be
+// moved over the wait.  __restrict__ is for tables that were complete before the chain.  A stream
+// under capture gets an ordinary launch, and so an ordinary graph edge.
 template <typename... P, typename... A>
 void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
   cudaLaunchAttribute attr{};

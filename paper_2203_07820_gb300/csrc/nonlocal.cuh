@@ -12,6 +12,9 @@
 // columns of 16 atoms at 176k DoFs: 26 us against 43; one FP64 column of one atom: 10.4 us against
 // 23.5, and 4 against 18 for the update below, whose lanes no longer idle.  100 FP64 columns of 6
 // atoms at 109k DoFs: coefficients and update 99 us against 104, on the FP64 pipe.
+//
+// X, Z and P are written by kernels that may still run when a CTA is placed (launch_after): plain loads,
+// no __restrict__.  The tables were complete before.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -45,7 +48,7 @@ struct F32x4 {
   using E = float; using V = float4; using W = double; using S = float;
   static constexpr int kCols = 4, kLanes = 32;
   static __device__ __forceinline__ V zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-  static __device__ __forceinline__ V load(const E* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+  static __device__ __forceinline__ V load(const E* p) { return *reinterpret_cast<const float4*>(p); }
   static __device__ __forceinline__ void mad(V& s, S w, V x) {
     s.x = fmaf(w, x.x, s.x); s.y = fmaf(w, x.y, s.y); s.z = fmaf(w, x.z, s.z); s.w = fmaf(w, x.w, s.w);
   }
@@ -102,7 +105,7 @@ struct Cplx {   // mad: conj(weight) x, madn: weight x
 // columns, 32 / LC entries at a time per warp.  Nodes and weights are in shared memory, so the
 // rows are the only loads and eight of them are in flight per lane.
 template <class T, int LC, int G>
-__device__ __forceinline__ void sums(typename T::V (&acc)[kNlGroup], const typename T::E* __restrict__ X, int64_t ldx,
+__device__ __forceinline__ void sums(typename T::V (&acc)[kNlGroup], const typename T::E* X, int64_t ldx,
                                      const int32_t* node, const typename T::S (*val)[kChunk], int len) {
   constexpr int EL = 32 / LC;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -116,10 +119,10 @@ __device__ __forceinline__ void sums(typename T::V (&acc)[kNlGroup], const typen
 
 template <class T, int LC>
 __global__ void __cluster_dims__(kSplits, 1, 1) __launch_bounds__(32 * kWarps)
-    k_nl_coef(const typename T::E* __restrict__ X, int64_t ldx, int ncol, const int32_t* __restrict__ group,
+    k_nl_coef(const typename T::E* X, int64_t ldx, int ncol, const int32_t* __restrict__ group,
               const int64_t* __restrict__ prow, const int32_t* __restrict__ pnode,
               const typename T::W* __restrict__ pval, const double* __restrict__ hcoup,
-              typename T::E* __restrict__ P, int64_t ldP) {
+              typename T::E* P, int64_t ldP) {
   using V = typename T::V;
   constexpr size_t kRed = sizeof(V) * kNlGroup * kWarps * LC, kVal = sizeof(typename T::S) * kNlGroup * kChunk;
   __shared__ alignas(16) uint8_t buf[kRed > kVal ? kRed : kVal];
@@ -184,11 +187,11 @@ __global__ void __cluster_dims__(kSplits, 1, 1) __launch_bounds__(32 * kWarps)
 // Z[node] += alpha sum_t w_t P[a_t] on the support nodes: LC lanes over columns per node, each row
 // of Z read before its projectors are walked
 template <class T, int LC>
-__global__ void __launch_bounds__(256) k_nl_add(typename T::E* __restrict__ Z, int64_t ldz, int ncol,
+__global__ void __launch_bounds__(256) k_nl_add(typename T::E* Z, int64_t ldz, int ncol,
                                                 const int32_t* __restrict__ snode, const int64_t* __restrict__ srow,
                                                 const int32_t* __restrict__ sproj,
                                                 const typename T::S* __restrict__ sval,
-                                                const typename T::E* __restrict__ P, int64_t ldP, int64_t nsup,
+                                                const typename T::E* P, int64_t ldP, int64_t nsup,
                                                 double alpha) {
   after_previous();
   const int64_t s = blockIdx.x * (int64_t)(256 / LC) + threadIdx.x / LC;

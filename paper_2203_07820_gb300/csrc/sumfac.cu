@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(SfCfg<W, N>::THREADS, SfCfg<W, N>::MINB)
     copy_commit();
     // scalars of the kernel's arithmetic: T, or float pairs (whose potential is stored as pairs)
     using E = std::conditional_t<PAIRS, sf::DF, T>;
-    E vv[N];                                              // the potential of this thread's z line
+    E vv[N];          // the potential of this thread's z line (plain loads: the kernel before may have formed it)
     {
       const E* v = reinterpret_cast<const E*>(it.v) + (int64_t)q.cell * (N * N * N) +
                    (NODAL ? (j * N + i) * N : j * N + i);
@@ -238,10 +238,10 @@ __global__ void __launch_bounds__(SfCfg<W, N>::THREADS, SfCfg<W, N>::MINB)
         vv[c] = E{};
         if (q.ok) {
           if constexpr (PAIRS) {
-            const float2 t = __ldg(reinterpret_cast<const float2*>(v + c * (NODAL ? 1 : N * N)));
+            const float2 t = *reinterpret_cast<const float2*>(v + c * (NODAL ? 1 : N * N));
             vv[c] = sf::DF{t.x, t.y};
           } else {
-            vv[c] = __ldg(v + c * (NODAL ? 1 : N * N));
+            vv[c] = v[c * (NODAL ? 1 : N * N)];
           }
         }
       }
