@@ -35,6 +35,8 @@ __device__ __forceinline__ double conj_of(double a) { return a; }
 __device__ __forceinline__ double2 conj_of(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double real_of(double a) { return a; }
 __device__ __forceinline__ double real_of(double2 a) { return a.x; }
+__device__ __forceinline__ bool is_real(double) { return true; }
+__device__ __forceinline__ bool is_real(double2 a) { return a.y == 0.0; }
 __device__ __forceinline__ double abs2(double a) { return a * a; }
 __device__ __forceinline__ double abs2(double2 a) { return fma(a.x, a.x, a.y * a.y); }
 __device__ __forceinline__ double add(double a, double b) { return a + b; }
@@ -136,12 +138,13 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(const C* __restrict__ A
     nrm = block_total<double, kTriThreads>(nrm, redd);      // |x below its first entry|^2
     if (b == 0 && threadIdx.x == 0) d[j] = real_of(x[j]);
     if (j == N - 1) break;
-    // reflector: H^H x = beta e_1, beta real
+    // reflector: H^H x = beta e_1, beta real (an entry with nothing below it may still need its phase
+    // taken out, however small its imaginary part: squares would round that away)
     const C a = x[j + 1];
     const double full = nrm + abs2(a);
     double beta = real_of(a);
     C inv = zero, tnew = zero;
-    if (nrm > 0.0 || abs2(a) > real_of(a) * real_of(a)) {
+    if (full > 0.0 && (nrm > 0.0 || !is_real(a))) {
       const double rs = real_of(a) > 0.0 ? -rsqrt(full) : rsqrt(full);      // 1 / beta
       beta = full * rs;
       if constexpr (sizeof(C) == 16) {                      // inv = 1 / (alpha - beta)

@@ -113,3 +113,34 @@ def test_beyond_the_shared_memory_rows(dg, box):
     g.manual_seed(1)
     X = torch.linalg.qr(torch.rand((M, 1900), generator=g, dtype=torch.float64, device="cuda") - 0.5)[0].contiguous()
     _check(dg, ham, X, False)
+
+
+def _unitary(N, blocks, eps, seed):
+    """R expm(i eps K), R real orthogonal and K real symmetric, both block diagonal in `blocks` (None:
+    one block): H^ = U^H diag(theta) U is real up to an imaginary part of about eps."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    U = torch.zeros((N, N), dtype=torch.complex128, device="cuda")
+    for s in range(0, N, blocks or N):
+        n = min(blocks or N, N - s)
+        R = torch.linalg.qr(torch.rand((n, n), generator=g, dtype=torch.float64, device="cuda") - 0.5)[0]
+        K = torch.rand((n, n), generator=g, dtype=torch.float64, device="cuda") - 0.5
+        U[s:s + n, s:s + n] = R.to(U.dtype) @ torch.linalg.matrix_exp(1j * eps * (K + K.t()))
+    return U
+
+
+@pytest.mark.parametrize("eps", [1e-8, 1e-9, 1e-10])
+@pytest.mark.parametrize("N,blocks", [(2, None), (3, None), (16, 2), (33, 2), (40, None), (65, None)])
+def test_weakly_complex_blocks(dg, box, N, blocks, eps):
+    """H^ whose imaginary part is eps of its real part, down to the couplings of decoupled 2 x 2
+    blocks, where nothing lies below the entry that a reflector makes real."""
+    ham, M, lam, V1 = box
+    e = (lam[:, None, None] + lam[None, :, None] + lam[None, None, :]).reshape(-1)
+    # one state of each level, so that every pair of columns is coupled
+    order = torch.argsort(e, stable=True)
+    first = torch.cat([torch.ones(1, dtype=torch.bool, device="cuda"), e[order].diff() > 1e-3])
+    idx = order[first][:N]
+    assert idx.numel() == N
+    q = V1.shape[0]
+    X = torch.einsum("zn,yn,xn->zyxn", V1[:, idx // (q * q)], V1[:, idx // q % q], V1[:, idx % q]).reshape(M, N)
+    _check(dg, ham, (X.to(torch.complex128) @ _unitary(N, blocks, eps, N)).contiguous(), True, e[idx])
