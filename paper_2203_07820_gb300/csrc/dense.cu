@@ -301,6 +301,7 @@ __global__ void k_bar_init(Barrier* b, long long limit, unsigned int missing) {
   b->reads = 0;
   b->limit = limit > 0 ? limit : (long long)kBarrierSpins;
   b->missing = missing;
+  b->top = 0;
 }
 void init_barrier(cudaStream_t s, Barrier* b, long long limit, unsigned int missing) {
   DFTFE_LAUNCH(k_bar_init, 1, 1, 0, s, b, limit, missing);

@@ -45,6 +45,8 @@ __device__ __forceinline__ double mul(double a, double b) { return a * b; }
 __device__ __forceinline__ double2 mul(double2 a, double2 b) {
   return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
+__device__ __forceinline__ double top_of(double a) { return fabs(a); }
+__device__ __forceinline__ double top_of(double2 a) { return fmax(fabs(a.x), fabs(a.y)); }
 __device__ __forceinline__ double scale(double s, double a) { return s * a; }
 __device__ __forceinline__ double2 scale(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
 // c + a b
@@ -75,6 +77,17 @@ template <typename C, int TT> __device__ __forceinline__ C block_total(C v, C* r
   return t;
 }
 
+// The matrix is scaled by the power of two that brings its largest entry to [1/2, 1): exact, and neither
+// the squares of the reflectors nor the thresholds of the divide and conquer, which are set against
+// vectors of norm one, depend on the unit of A.  Biased exponent of that power from the bits of the
+// largest entry (a matrix of zeros, or one that is not finite, is left alone; the ends of the range are
+// drawn in, so that the power and its reciprocal are normal numbers).
+__device__ __forceinline__ int scale_exponent(unsigned long long top) {
+  const int e = (int)(top >> 52);
+  return top == 0 || e == 2047 ? 1023 : min(max(2045 - e, 1), 2044);
+}
+__device__ __forceinline__ double pow2(int biased) { return __longlong_as_double((long long)biased << 52); }
+
 // -------------------------------------------------------- tridiagonalisation
 constexpr int kTriThreads = 128;    // one warp per sub-partition: scalar steps repeat in all of them for free
 // Rows i = blockIdx.x, blockIdx.x + gridDim.x, ... of A (lower triangle read) live in shared
@@ -98,16 +111,26 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(const C* __restrict__ A
   C* const x = w + N;                                       // pivot row, then the new reflector
   const C zero = zero_of(C());
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long top = 0;                // as bits: non-negative doubles order alike, NaN above all
   for (int r = 0; r < nrow; ++r) {
     const int i = b + r * G;
-    for (int k = threadIdx.x; k < N; k += kTriThreads)
-      rows[(size_t)r * N + k] = k <= i ? A[(size_t)i * N + k] : conj_of(A[(size_t)k * N + i]);
+    for (int k = threadIdx.x; k < N; k += kTriThreads) {
+      const C t = k <= i ? A[(size_t)i * N + k] : conj_of(A[(size_t)k * N + i]);
+      rows[(size_t)r * N + k] = t;
+      top = max(top, (unsigned long long)__double_as_longlong(top_of(t)));
+    }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if (lane == 0 && top) atomicMax(&bar->top, top);
   for (int k = threadIdx.x; k < N; k += kTriThreads) v[k] = w[k] = zero;
   __syncthreads();
   if (b == 0)
     for (int k = threadIdx.x; k < N; k += kTriThreads) xr[N + k] = rows[k];     // read as column -1's
   if (!jac::grid_barrier(bar, status)) return;
+  const double sc = pow2(scale_exponent(__ldcg(&bar->top)));
+  for (int t = threadIdx.x; t < nrow * N; t += kTriThreads) rows[t] = scale(sc, rows[t]);
+  __syncthreads();
   C tau = zero;
   for (int j = 0; j < N; ++j) {
     const int cur = j & 1, old = cur ^ 1;
@@ -131,7 +154,8 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(const C* __restrict__ A
     double nrm = 0.0;
     for (int k = j + threadIdx.x; k < N; k += kTriThreads) {
       C r = __ldcg(ro + k);
-      if (j > 0) r = mad(neg(vj), conj_of(w[k]), mad(neg(wj), conj_of(v[k]), r));
+      if (j == 0) r = scale(sc, r);
+      else r = mad(neg(vj), conj_of(w[k]), mad(neg(wj), conj_of(v[k]), r));
       x[k] = conj_of(r);
       if (k > j + 1) nrm += abs2(r);
     }
@@ -139,12 +163,13 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(const C* __restrict__ A
     if (b == 0 && threadIdx.x == 0) d[j] = real_of(x[j]);
     if (j == N - 1) break;
     // reflector: H^H x = beta e_1, beta real (an entry with nothing below it may still need its phase
-    // taken out, however small its imaginary part: squares would round that away)
+    // taken out, however small its imaginary part: squares would round that away).  Entries below
+    // 1e-140 of the largest one count as zeros, so that their squares stay in range.
     const C a = x[j + 1];
     const double full = nrm + abs2(a);
     double beta = real_of(a);
     C inv = zero, tnew = zero;
-    if (full > 0.0 && (nrm > 0.0 || !is_real(a))) {
+    if (full > 1e-280 && (nrm > 0.0 || !is_real(a))) {
       const double rs = real_of(a) > 0.0 ? -rsqrt(full) : rsqrt(full);      // 1 / beta
       beta = full * rs;
       if constexpr (sizeof(C) == 16) {                      // inv = 1 / (alpha - beta)
@@ -715,13 +740,16 @@ __device__ __forceinline__ void sum4(double2 (&s)[4]) {
 }
 
 // z <- H_0 (H_1 (... z)) for one eigenvector per warp: Z row (real, N) -> out row (N); the vector stays
-// in registers (lane l holds components l + 32 q), the reflectors stream from L2.
+// in registers (lane l holds components l + 32 q), the reflectors stream from L2.  The eigenvalues go
+// back to the matrix's scale here.
 template <typename C, int E>
 __global__ void __launch_bounds__(64) k_backtransform(const double* __restrict__ Z, const C* __restrict__ V,
                                                       const C* __restrict__ tri, int N, int nref,
-                                                      C* __restrict__ out) {
+                                                      C* __restrict__ out, const jac::Barrier* __restrict__ bar,
+                                                      double* __restrict__ d) {
   const int lane = threadIdx.x & 31, i = blockIdx.x * 2 + (threadIdx.x >> 5);
   if (i >= N) return;
+  if (lane == 0) d[i] *= pow2(2046 - scale_exponent(bar->top));
   C z[E];
 #pragma unroll
   for (int q = 0; q < E; ++q) {
@@ -779,8 +807,9 @@ template <typename C> static size_t tri_smem(int N, int G) {
 }
 
 template <typename C, int E>
-static void launch_back(cudaStream_t s, const double* Z, const C* V, const C* tri, int N, int nref, C* out) {
-  DFTFE_LAUNCH((k_backtransform<C, E>), (unsigned)((N + 1) / 2), 64, 0, s, Z, V, tri, N, nref, out);
+static void launch_back(cudaStream_t s, const Dc& w, const C* V, const C* tri, int nref, C* out,
+                        const jac::Barrier* bar) {
+  DFTFE_LAUNCH((k_backtransform<C, E>), (unsigned)((w.N + 1) / 2), 64, 0, s, w.Qa, V, tri, w.N, nref, out, bar, w.d);
 }
 
 }  // namespace eig
@@ -867,12 +896,12 @@ void tridiag_eig(dftfe_ham h, const C* A, int N, double* d, C* VT, int* d_status
   }
   DFTFE_LAUNCH(k_wy<C>, (unsigned)((nref + 3) / 4), 32, 0, st, V, tau, N, nref, tri);
   const int E = (N + 31) / 32;
-  if (E <= 2) launch_back<C, 2>(st, w.Qa, V, tri, N, nref, VT);
-  else if (E <= 4) launch_back<C, 4>(st, w.Qa, V, tri, N, nref, VT);
-  else if (E <= 8) launch_back<C, 8>(st, w.Qa, V, tri, N, nref, VT);
-  else if (E <= 16) launch_back<C, 16>(st, w.Qa, V, tri, N, nref, VT);
-  else if (E <= 32) launch_back<C, 32>(st, w.Qa, V, tri, N, nref, VT);
-  else if constexpr (sizeof(C) == 8) launch_back<C, 64>(st, w.Qa, V, tri, N, nref, VT);
+  if (E <= 2) launch_back<C, 2>(st, w, V, tri, nref, VT, bar);
+  else if (E <= 4) launch_back<C, 4>(st, w, V, tri, nref, VT, bar);
+  else if (E <= 8) launch_back<C, 8>(st, w, V, tri, nref, VT, bar);
+  else if (E <= 16) launch_back<C, 16>(st, w, V, tri, nref, VT, bar);
+  else if (E <= 32) launch_back<C, 32>(st, w, V, tri, nref, VT, bar);
+  else if constexpr (sizeof(C) == 8) launch_back<C, 64>(st, w, V, tri, nref, VT, bar);
 }
 template void tridiag_eig<double>(dftfe_ham, const double*, int, double*, double*, int*);
 template void tridiag_eig<double2>(dftfe_ham, const double2*, int, double*, double2*, int*);

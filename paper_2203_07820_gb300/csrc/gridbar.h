@@ -17,6 +17,7 @@ struct Barrier {
   unsigned int reads;   // CTAs that have read the rotation inputs, summed over rounds
   long long limit;      // spin iterations before a wait gives up
   unsigned int missing; // arrivals the barrier expects beyond the grid (0; 1 only in the wait test)
+  unsigned long long top;   // bits of the largest |entry| of the matrix (k_tridiag)
 };
 
 // every call starts from a cleared barrier with its spin limit and expected arrivals (dense.cu)

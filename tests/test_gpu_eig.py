@@ -144,3 +144,34 @@ def test_weakly_complex_blocks(dg, box, N, blocks, eps):
     q = V1.shape[0]
     X = torch.einsum("zn,yn,xn->zyxn", V1[:, idx // (q * q)], V1[:, idx // q % q], V1[:, idx % q]).reshape(M, N)
     _check(dg, ham, (X.to(torch.complex128) @ _unitary(N, blocks, eps, N)).contiguous(), True, e[idx])
+
+
+@pytest.mark.parametrize("cplx", [False, True])
+@pytest.mark.parametrize("power", [13, 25, 300, -20, -300])
+def test_the_scale_of_the_operator_does_not_matter(dg, box, power, cplx):
+    """An empty box 2^power times as long: H~ is 2^(-2 power) times that of the small box, to the last
+    bit, and so are the Ritz values; the vectors are the same."""
+    ham, M, lam, V1 = box
+    N = 72
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    X = torch.rand((M, N, 2), generator=g, dtype=torch.float64, device="cuda") - 0.5
+    X = torch.linalg.qr(torch.view_as_complex(X) if cplx else X[:, :, 0])[0].contiguous()
+    mesh2 = dg.dftfe_mesh_create(5.0 * 2.0 ** power, 6, 3)
+    ham2 = dg.dftfe_ham_create(mesh2)
+    try:
+        _, ncell, _, nq = dg.dftfe_mesh_info(mesh2)
+        dg.dftfe_ham_set_potential(ham2, torch.zeros(ncell * nq, dtype=torch.float64, device="cuda"))
+        dg.dftfe_ham_set_kpoint(ham2, (0.0, 0.0, 0.0))
+        out = []
+        for h in (ham, ham2):
+            Y, HY, ev = X.clone(), torch.empty_like(X), torch.empty(N, dtype=torch.float64, device="cuda")
+            (dg.dftfe_rayleigh_ritz_z if cplx else dg.dftfe_rayleigh_ritz)(h, Y, ev, HY)
+            out.append((Y, HY, ev))
+        torch.cuda.synchronize()
+        (Y, HY, ev), (Y2, HY2, ev2) = out
+        assert torch.equal(ev2 * 4.0 ** power, ev)
+        assert torch.equal(Y2, Y) and torch.equal(HY2 * 4.0 ** power, HY)
+    finally:
+        dg.dftfe_ham_destroy(ham2)
+        dg.dftfe_mesh_destroy(mesh2)
