@@ -178,3 +178,55 @@ def test_projectors_on_common_supports(dg, ncol):
             assert np.all(np.abs(got[0] - got[1]) <= 448 * u * zbound + 4 * u * np.abs(got[0])), prec
     finally:
         _destroy(dg, mesh, ham)
+
+
+@pytest.mark.parametrize("vquad", [0, 1])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_pairs_keep_non_finite_entries(dg, bad, vquad):
+    """A NaN or an infinity in the block or in the potential reaches every entry of the FP64-accurate
+    products that it makes non-finite in FP64; the other columns, and without column scaling the
+    other rows, stay right."""
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 6.5), (3, 2, 4), 4, vquad)
+    try:
+        X = torch.from_numpy(synth.random_block(7, om.ndofs, 5)).cuda()
+        row = om.ndofs // 3
+        Xbad = X.clone()
+        Xbad[row, 2] = bad
+        _, ncell, _, nq = dg.dftfe_mesh_info(mesh)
+        v = torch.from_numpy(synth.random_block(9, ncell * nq, 1)).cuda().reshape(-1)
+        vbad = v.clone()
+        vbad[v.numel() // 2] = bad
+        for pot, x in ((v, Xbad), (vbad, X)):
+            dg.dftfe_ham_set_potential(ham, pot)
+            ref = torch.empty_like(X)
+            dg.dftfe_ham_apply(ham, x, ref)
+            lost = ~torch.isfinite(ref)
+            assert lost.any()
+            for prec in (dg.DFTFE_FP64_FLOAT_PAIRS, dg.DFTFE_FP64_SLICES):
+                Y = torch.zeros_like(X)
+                dg.dftfe_ham_apply(ham, x, Y, prec)
+                assert not torch.isfinite(Y[lost]).any(), prec
+                keep = ~lost
+                if prec == dg.DFTFE_FP64_SLICES and x is Xbad:
+                    keep = keep & (torch.arange(5, device="cuda") != 2)
+                assert (Y - ref)[keep].abs().max().item() <= 1e-12 * ref[keep].abs().max().item(), prec
+    finally:
+        _destroy(dg, mesh, ham)
+
+
+def test_pairs_beyond_the_range_of_fp32(dg):
+    """Entries above 2^128: the scaled form keeps them, the unscaled one has no representation for them and
+    says so."""
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 6.5), (3, 2, 4), 4)
+    try:
+        X = torch.from_numpy(synth.random_block(7, om.ndofs, 5)).cuda()
+        for scale in (2.0 ** 140, 2.0 ** 900):
+            x = X * scale
+            ref, Y = torch.empty_like(X), torch.empty_like(X)
+            dg.dftfe_ham_apply(ham, x, ref)
+            dg.dftfe_ham_apply(ham, x, Y, dg.DFTFE_FP64_SLICES)
+            assert (Y - ref).abs().max().item() <= TOL * ref.abs().max().item()
+            dg.dftfe_ham_apply(ham, x, Y, dg.DFTFE_FP64_FLOAT_PAIRS)
+            assert not torch.isfinite(Y).any()
+    finally:
+        _destroy(dg, mesh, ham)
