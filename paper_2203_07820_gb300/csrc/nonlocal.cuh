@@ -229,6 +229,7 @@ void coef(dftfe_ham h, cudaStream_t stream, const typename T::E* X, int64_t ldx,
 template <class T>
 void add(dftfe_ham h, cudaStream_t stream, typename T::E* Z, int64_t ldz, int ncol, const typename T::S* sval,
          const typename T::E* P, int64_t ldP, double alpha) {
+  if (h->nsup == 0) return;      // every support is empty: the term is zero, and so would be the grid
   if constexpr (T::kCols == 1) {
     if (ncol == 1) {
       launch_after(k_nl_add<T, 1>, (unsigned)((h->nsup + 255) / 256), 256, 0, stream, Z, ldz, ncol, h->d_snode,

@@ -230,3 +230,28 @@ def test_pairs_beyond_the_range_of_fp32(dg):
             assert not torch.isfinite(Y).any()
     finally:
         _destroy(dg, mesh, ham)
+
+
+def test_projectors_with_empty_supports_add_nothing(dg):
+    om, oh, mesh, ham = _system(dg, (5.0, 4.0, 4.0), (3, 2, 2), 4)
+    try:
+        X = torch.from_numpy(synth.random_block(5, om.ndofs, 6)).cuda()
+        bounds = dg.dftfe_spectrum_bounds(ham, 10, 1, 6)
+
+        def results():
+            out = []
+            for prec in (dg.DFTFE_FP64, dg.DFTFE_MIXED_TF32X3, dg.DFTFE_FP64_FLOAT_PAIRS):
+                Y = torch.full_like(X, float("nan"))
+                dg.dftfe_ham_apply(ham, X, Y, prec)
+                out.append(Y)
+            Y = X.clone()
+            dg.dftfe_chebyshev_filter(ham, Y, 5, bounds, dg.DFTFE_MIXED_TF32X3)
+            return out + [Y]
+
+        without = results()
+        dg.dftfe_ham_set_nonlocal(ham, np.array([0.5, 0.7]), np.zeros(3, dtype=np.int64), np.zeros(0, dtype=np.int64),
+                                  np.zeros(0))
+        for a, b in zip(without, results()):
+            assert torch.equal(a, b)
+    finally:
+        _destroy(dg, mesh, ham)
