@@ -29,6 +29,12 @@ def sources():
     return sorted(f for f in os.listdir(CSRC) if f.endswith((".cu", ".cc")))
 
 
+def dependencies():
+    """Every file the library is built from: sources, headers (device code in .cuh among them), the ABI."""
+    return [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC)) if f.endswith((".cu", ".cc", ".h", ".cuh"))] + [
+        os.path.join(os.path.dirname(HERE), "include", "dftfe_gb300.h")]
+
+
 def _compile(src, verbose):
     obj = os.path.join(BUILD, os.path.splitext(src)[0] + ".o")
     cmd = [nvcc(), *ARCH, *FLAGS, "-x", "cu" if src.endswith(".cu") else "c++",
@@ -48,11 +54,8 @@ def _compile(src, verbose):
 def build(verbose=False, force=False):
     os.makedirs(BUILD, exist_ok=True)
     srcs = sources()
-    deps = [os.path.join(CSRC, s) for s in srcs] + [
-        os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC)) if f.endswith(".h")] + [
-        os.path.join(os.path.dirname(HERE), "include", "dftfe_gb300.h")]
     if (not force and os.path.exists(LIB)
-            and os.path.getmtime(LIB) >= max(os.path.getmtime(d) for d in deps)):
+            and os.path.getmtime(LIB) >= max(os.path.getmtime(d) for d in dependencies())):
         return LIB
     with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
         results = list(ex.map(lambda s: _compile(s, verbose), srcs))
