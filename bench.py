@@ -7,8 +7,9 @@ p = 6 GLL elements (343 nodes/cell, 192^3 = 7,077,888 DoFs), 64 Gaussian wells
 Gaussian radial width 1 bohr, cutoff 3 bohr, couplings U[0.5, 2] Ha); 1,024 states,
 block 128, Chebyshev degree 40.  A step is one pass: filter (8 blocks x 40
 applications of H~), Cholesky-Gram-Schmidt, Rayleigh-Ritz, residuals, bounds update,
-with the filter's cell products as 3-term TF32 splits (FP32 accumulation) and
-Cholesky, eigensolver and residuals in FP64.
+with the filter's operator as FP32 1D contractions, overlap, projection and rotations as
+three-slice TF32 products off their FP64 diagonals, W = H~X in float pairs, and Cholesky,
+eigensolver and residuals in FP64.
 
 The FP64 arm of the comparison is one CUDA-event-timed FP64 pass from the same state
 (`mixed_vs_fp64`), with the Ritz values of both and the generalised residual of the
@@ -69,8 +70,8 @@ def describe(wl):
             "ndofs": wl.ndofs, "nstates": wl.nstates, "block": wl.block,
             "cheb_degree": wl.cheb_degree, "atoms": int(wl.centres.shape[0]), "projectors": wl.nproj,
             "seed": wl.seed,
-            "l2": f"inputs larger than L2 (FP32 cell matrices {wl.ncell ** 3 * (wl.degree + 1) ** 6 * 4 / 1e9:.2f} GB"
-                  " streamed per H~X)"}
+            "l2": f"inputs larger than L2 (X {wl.ndofs * wl.nstates * 8 / 1e9:.2f} GB; in the FP32 filter three blocks of"
+                  f" {wl.ndofs * wl.block * 4 / 1e9:.2f} GB read or written per H~X)"}
 
 
 # ----------------------------------------------------------------- clocks
@@ -293,8 +294,8 @@ def kpoint_step(dg, dev, stream, steps=2, warmup=1):
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
     roofs = {}
     if "cell_gemm_fp64" in fam:
-        # the real cell products act on the real view: 2 real columns per complex column
-        a = 2.0 * Nc * nc * nc * 2 * apps / (fam["cell_gemm_fp64"]["ms"] / 1e3) / 1e12
+        # the real operator acts on the real view: 2 real columns per complex column
+        a = 18.0 * Nc * nc * (p + 1) * 2 * apps / (fam["cell_gemm_fp64"]["ms"] / 1e3) / 1e12
         roofs["cell_gemm_fp64"] = {"bound": "alu", "achieved": a, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                                    "frac": a / FP64_PEAK_TFLOPS}
     if "kin_k" in fam:
@@ -322,7 +323,7 @@ def kpoint_step(dg, dev, stream, steps=2, warmup=1):
     torch.cuda.synchronize()
     spp_tg = e0.elapsed_time(e1) / 1e3 / steps
     rows, best_ms, heur_ms = dg.dftfe_autotune_query(ham, 2 * blk)
-    # the complex64 form (TF32x3 split cell products, FP32 complex vectors; CholGS / RR mixed on
+    # the complex64 form (FP32 1D contractions and complex vectors; CholGS / RR mixed on
     # the real view, W from float pairs), and its Ritz values against a complex128 pass taken
     # from the same state
     X.copy_(X0)
@@ -350,7 +351,7 @@ def kpoint_step(dg, dev, stream, steps=2, warmup=1):
            "dtype": "c128 (FP64)",
            "s_per_pass_autotuned_graphed": spp_tg,
            "autotune": {"rows_per_cta": rows, "best_ms": best_ms, "heuristic_ms": heur_ms,
-                        "note": "one FP64 cell-product pass over the mesh on 2 x block real columns; "
+                        "note": "one FP64 pass of the local operator over the mesh on 2 x block real columns; "
                                 "rows_per_cta 0 = the built-in heuristic"},
            "graph_replays": dg.dftfe_graph_query(ham)[0],
            "s_per_pass_c64_tf32x3": spp_c64,
@@ -437,14 +438,14 @@ def batch_kpoint_step(dg, dev, stream, seed=0, systems=None):
         run_batch(batch, items, P32)                                  # first graphed shape runs directly
         t_graphed = run_batch(batch, items, P32)
         replays = dg.dftfe_batch_graph_query(batch)[0]
-        # algorithmic split-precision filter flops: 3 products x 2 N_c n_c^2 per real column
-        flops = sum(3.0 * 2.0 * it["wl"].ncell ** 3 * (it["wl"].degree + 1) ** 6 * 2 * it["wl"].nstates *
+        # filter flops: nine 1D contractions, 18 N_c n_c (p + 1) per real column and application
+        flops = sum(18.0 * it["wl"].ncell ** 3 * (it["wl"].degree + 1) ** 4 * 2 * it["wl"].nstates *
                     it["wl"].cheb_degree for it in items)
         out["c64_tf32x3"] = {
             "s_per_pass": t_plain, "s_per_pass_autotuned": t_tuned, "s_per_pass_autotuned_graphed": t_graphed,
             "s_tuning_pass": t_tune_first, "graph_replays": replays,
             "phases_ms_per_pass": {k: v for k, v in fam.items()},
-            "filter_tflops_split_products": flops / (fam["batch_filter"] / 1e3) / 1e12 if fam["batch_filter"] else None,
+            "filter_tflops": flops / (fam["batch_filter"] / 1e3) / 1e12 if fam["batch_filter"] else None,
             "autotune": tuned,
             "max_resid": max(float(it["rs"].max().item()) for it in items)}
     finally:
@@ -943,7 +944,9 @@ def run_ours(args, rank, world, local, tdist):
 
     nc = (wl.degree + 1) ** 3
     Nc = wl.ncell ** 3
-    filter_flops = 2.0 * Nc * nc * nc * N * wl.cheb_degree          # algorithmic, per pass
+    # per pass: the operator as its nine 1D contractions (BF16x3: as its dense cell products)
+    contraction_flops = 18.0 * Nc * nc * (wl.degree + 1) * N * wl.cheb_degree
+    filter_flops = 2.0 * Nc * nc * nc * N * wl.cheb_degree if args.precision == "bf16x3" else contraction_flops
     t_filter = fam.get("pass_filter", {}).get("ms", float("nan")) / 1e3
     roofs = rooflines(fam, wl, args.precision)
     timed = {k: v["ms"] for k, v in fam.items() if not k.startswith("pass_") and k in roofs}
@@ -1008,7 +1011,7 @@ def run_ours(args, rank, world, local, tdist):
         h2 = N // 2
         conv = rg <= 1e-5
         compare = {"fp64_pass_s": t64, "fp64_phases_ms": {k: v["ms"] for k, v in fam64.items()},
-                   "fp64_filter_tflops": filter_flops / (fam64["pass_filter"]["ms"] / 1e3) / 1e12
+                   "fp64_filter_tflops": contraction_flops / (fam64["pass_filter"]["ms"] / 1e3) / 1e12
                    if "pass_filter" in fam64 else None,
                    "speedup_mixed_over_fp64": t64 / sec_per_pass,
                    "max_abs_deps_Ha": float(d.max().item()),
@@ -1070,7 +1073,9 @@ def run_ours(args, rank, world, local, tdist):
         torch.cuda.synchronize()
         dens = {"split_rr_and_fermi_ms": d0.elapsed_time(d1), "density_ms": d1.elapsed_time(d2),
                 "nfr": nfr, "mu_Ha": mu, "kT_Ha": kT,
-                "density_fp64_tflops": 2.0 * Nc * (wl.degree + 1) ** 6 * (N + nfr) / (d1.elapsed_time(d2) / 1e3) / 1e12}
+                # three 1D contractions and the weighted square per column
+                "density_fp64_tflops": Nc * nc * (6.0 * (wl.degree + 1) + 3.0) * (N + nfr)
+                / (d1.elapsed_time(d2) / 1e3) / 1e12}
         del Xfr, rho
       except Exception as exc:            # a side measurement must not hide the main one
         dens = {"error": repr(exc)}
