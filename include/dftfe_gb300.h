@@ -63,7 +63,8 @@ typedef enum {
                               relative per product).  CholGS and Rayleigh-Ritz as below */
   DFTFE_FP64_FLOAT_PAIRS = 3, /* dftfe_ham_apply(_z) only: FP64-accurate local operator from
                               pairs of floats (error-free products, TwoSum accumulation, about
-                              44 significant bits) on the FP32 pipes; FP64 in and out */
+                              44 significant bits) on the FP32 pipes; FP64 in and out, entries
+                              inside FP32's range (beyond it NaN) */
   DFTFE_FP64_SLICES = 4     /* dftfe_ham_apply(_z) only: FP64-accurate local operator; default
                               and nodal rules: float-pair 1D contractions of columns scaled by
                               their largest entry's exponent; other rules: cell products on
@@ -245,8 +246,8 @@ dftfe_status dftfe_random_uniform(double* out, int64_t n, uint64_t seed,
 /* k-step Lanczos with full reorthogonalisation on H~ (a7; the paper only says
  * the degree follows the upper bound of H~, Sec. 3.1).  v0: DEVICE start vector
  * (M doubles) or NULL to use dftfe_random_uniform(seed, offset 0).  Writes to
- * HOST out3 = {theta_min, theta_max, b}, b = theta_max + |beta_k| |s_k| (a
- * Ritz-residual upper bound).  Synchronises the stream. */
+ * HOST out3 = {theta_min, theta_max, b}, b = theta_max + |beta_k| (Zhou and Saad's
+ * upper bound).  Synchronises the stream. */
 dftfe_status dftfe_lanczos(dftfe_ham ham, int k, const double* v0, uint64_t seed,
                            double* out3);
 

@@ -7,7 +7,7 @@
 //
 // Layout: a complex block is complex128 DoF-major (real and imaginary parts interleaved), so
 // its real view is an M x 2 ncol FP64 block.  H~_loc is real: it acts on that real view as on
-// 2 ncol real columns, through the same FP64 cell products as at the Gamma point.
+// 2 ncol real columns, through the same kernels as at the Gamma point.
 //
 // The k.grad term is separable on the structured periodic mesh: with GLL quadrature on the
 // nodes, G_d is the 1D periodic derivative matrix G1_d (entries int l_a l_b' = w_a l_b'(x_a),
@@ -15,8 +15,8 @@
 // Loewdin scaling cancels those, so G~_d = G~1_d along axis d with G~1_d = m_d^-1/2 G1_d
 // m_d^-1/2.  A stencil kernel applies it (p+1 neighbours per axis inside an element, 2p+1
 // on element faces), fused with the recurrence terms.  Dense complex cell matrices (the
-// paper's form) would make every cell product four real FP64 products; here the cell
-// products stay real and the k-dependent part costs 3 (p+2) complex-by-real multiply-adds
+// paper's form) would make every cell product four real FP64 products; here the local
+// operator stays real and the k-dependent part costs 3 (p+2) complex-by-real multiply-adds
 // per entry on average (the kernel is bound by GB300's FP64 pipe, not by HBM).
 //
 // CholGS and Rayleigh-Ritz work on the real view.  With Xr the real view of X (M x 2N), the

@@ -1,5 +1,6 @@
-// Tensor-product form of H~_loc X (see sumfac.h): the FP64 cell kernel, the assembly of the
-// shared faces, and their launches for one system and for the batched passes.
+// Tensor-product form of H~_loc X (see sumfac.h): the cell kernel (FP64, FP32 and float pairs), the sums
+// over shared faces, their launches for one system and for the batched passes, and the density
+// at the quadrature points by the same contractions.
 #include "internal.h"
 #include "sumfac.h"
 #include "tcgen05.h"
@@ -914,7 +915,8 @@ void sf_local64(dftfe_ham h, const double* X, int64_t ldx, const double* Xp, int
 }
 
 // Y = H~_loc X from float pairs (FP64 blocks; about 2^-44 |H~||X|); ex: biased exponents of the columns'
-// largest entries, by which they are scaled on the way (NULL: the entries lie well inside FP32's range)
+// largest entries, by which they are scaled on the way (NULL: the entries lie well inside FP32's range;
+// above it they come out as NaN)
 void sf_local_pairs(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t ldy, int ncol, const int* ex) {
   auto* m = h->mesh;
   dftfe_ham o = loc(h);
