@@ -531,7 +531,7 @@ bool apply_slices(dftfe_ham h, const double* X, int64_t ldx, double* Y, int64_t 
   if (sf_applicable(m)) {
     // float pairs through the 1D contractions, each column scaled by its largest entry's power of two:
     // 48 bits relative to the column where the digits keep 41, no cell matrices to cut or stream (12^3
-    // cells, p = 6, 256 columns: 5.07 ms against 6.34, error 3.1e-15 against 3.6e-12)
+    // cells, p = 6, 256 columns: 4.98 ms against 6.34, error 3.1e-15 against 3.6e-12)
     int* ex = (int*)ws_get(h, "slices_xe", sizeof(int) * (size_t)std::max(ncol, (int)kBlk));
     DFTFE_CHECK_CUDA(cudaMemsetAsync(ex, 0, sizeof(int) * (size_t)std::max(ncol, (int)kBlk), h->stream));
     const unsigned gx = (unsigned)std::max(1, h->sm_count) * 4;

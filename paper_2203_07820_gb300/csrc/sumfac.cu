@@ -29,23 +29,32 @@ __device__ __forceinline__ int load_item(sf::Item<T>& it, const sf::Item<T>& one
 // FP64 -> float pair and back with integer operations (one FP64 subtraction or addition each).
 // As tc::narrow_f64, but magnitudes of 2^128 and more, infinities and NaNs among them, are held at
 // 2^128's exponent, which FP32 reads as infinity or NaN (the clamp is one operation of the nine).  Every
-// sum and product keeps that in the leading part, and it comes back as NaN.  W of 373,248 DoFs x 256
-// columns: 5.07 ms, 4.97 when such entries came out as ordinary numbers.
+// sum and product keeps that in the leading part, and it comes back as NaN.  The shifts and range
+// tests are written for few operations: W of 373,248 DoFs x 256 columns 4.97 ms, as without the tests;
+// with a test on each output beside tc::widen_f32 5.07 to 5.29.
 __device__ __forceinline__ float narrow_held(double x) {
   const int hi = __double2hiint(x), t = (hi & 0x7fffffff) - 0x38000000;      // exponent 897: FP32's smallest normal
   const uint32_t lo = (uint32_t)__double2loint(x);
   const uint32_t f = __funnelshift_l(lo, (uint32_t)min(t, 0x0ff00000), 3) + ((lo >> 28) & 1u);
   return __uint_as_float((t < 0x100000 ? 0u : f) | ((uint32_t)hi & 0x80000000u));
 }
+// exact widening (sign and exponent moved by one arithmetic shift); FP32 subnormals become (next to)
+// zero, exponent 255 is taken as 2^128
+__device__ __forceinline__ double widen_held(float f) {
+  const uint32_t u = __float_as_uint(f);
+  const int h = (((int)u >> 3) & (int)0x8fffffff) + 0x38000000;
+  return __hiloint2double((u & 0x7f800000u) ? h : 0, (int)(u << 29));
+}
 __device__ __forceinline__ sf::DF to_pair(double x) {
   const float hi = narrow_held(x);
-  return sf::DF{hi, narrow_held(x - tc::widen_f32(hi))};
+  return sf::DF{hi, narrow_held(x - widen_held(hi))};
 }
 __device__ __forceinline__ double from_pair(sf::DF a) {
-  const uint32_t u = __float_as_uint(a.hi), m = u & 0x7fffffffu;
-  // a normal entry, or zero, or NaN from exponent 255
-  const uint32_t h = m - 0x00800000u < 0x7f000000u ? (m >> 3) + 0x38000000u : m | (m >> 8);
-  return __hiloint2double((int)(h | (u & 0x80000000u)), (int)(u << 29)) + tc::widen_f32(a.lo);
+  const uint32_t u = __float_as_uint(a.hi);
+  const int h = (((int)u >> 3) & (int)0x8fffffff) + 0x38000000;
+  // a normal entry; otherwise zero, or NaN from exponent 255
+  const int w = (u << 1) - 0x01000000u < 0xfe000000u ? h : (int)(u << 1) >> 5;
+  return __hiloint2double(w, (int)(u << 29)) + widen_held(a.lo);
 }
 // For a column whose largest entry has biased exponent e (0: an all-zero column): 2^(e - 1022), its
 // scale, or with -e the reciprocal (the ends of the range drawn in, so that both are normal numbers).
